@@ -75,6 +75,9 @@ struct qd_reg {
     size_t red_cap = 0;     // doubles
     double *cdf = nullptr;  // lazily allocated N doubles
     double *cdf_chunks = nullptr;
+    double *samp = nullptr;    // lazily allocated prefix sums of qd_sample
+    void *shot = nullptr;      // device copies of a call's draws (and uniforms)
+    size_t shot_cap = 0;       // bytes
     int32_t *dev_err = nullptr;
     int64_t tile_stride = -1;  // -1: process default
     int32_t fuse_kmax = 3;     // largest number of qudits of a fused block
@@ -697,6 +700,8 @@ int qd_destroy(qd_reg *r) {
     if (r->red) cudaFree(r->red);
     if (r->cdf) cudaFree(r->cdf);
     if (r->cdf_chunks) cudaFree(r->cdf_chunks);
+    if (r->samp) cudaFree(r->samp);
+    if (r->shot) cudaFree(r->shot);
     if (r->dev_err) cudaFree(r->dev_err);
     delete r;
     return QD_OK;
@@ -1494,9 +1499,8 @@ int qd_norm(qd_reg *r, double *out) {
     if (int rc = reg_ok(r)) return rc;
     if (!out) return fail(QD_ERR_ARG, "null output");
     const int nb = reduce_blocks(r->sm_count);
-    Expand64 ex{};
     double *res = r->red + nb * 64;
-    QD_CUDA(slice_norms(r->psi, r->prec, (uint64_t)r->N, ex, 0, 1, r->red, nb, res, r->stream));
+    QD_CUDA(digit_norms(r->psi, r->prec, (uint64_t)r->N, (uint64_t)r->N, 1, r->red, nb, res, r->stream));
     QD_CUDA(cudaMemcpyAsync(out, res, sizeof(double), cudaMemcpyDeviceToHost, r->stream));
     QD_CUDA(cudaStreamSynchronize(r->stream));
     return QD_OK;
@@ -1527,10 +1531,8 @@ int qd_marginal(qd_reg *r, int32_t q, double *out) {
     if (q < 0 || q >= r->n) return fail(QD_ERR_ARG, "qudit out of range");
     const int nb = reduce_blocks(r->sm_count);
     const int d = r->dims[q];
-    Expand64 ex{};
-    set_expand64(ex, {{r->s[q], d}});
     double *res = r->red + (size_t)nb * 64;
-    QD_CUDA(slice_norms(r->psi, r->prec, (uint64_t)(r->N / d), ex, (uint64_t)r->s[q], d, r->red, nb, res, r->stream));
+    QD_CUDA(digit_norms(r->psi, r->prec, (uint64_t)r->N, (uint64_t)r->s[q], d, r->red, nb, res, r->stream));
     QD_CUDA(cudaMemcpyAsync(out, res, sizeof(double) * d, cudaMemcpyDeviceToHost, r->stream));
     QD_CUDA(cudaStreamSynchronize(r->stream));
     return QD_OK;
@@ -1564,26 +1566,49 @@ int qd_cdf(qd_reg *r, double *out, int32_t where) {
     return QD_OK;
 }
 
+constexpr size_t kShotKeep = size_t(1) << 24;  // 1 to 2 million shots
+
 static int sample_impl(qd_reg *r, const double *u_host, uint64_t seed, int64_t shots, int64_t *out) {
     if (int rc = reg_ok(r)) return rc;
     if (!out || shots < 0) return fail(QD_ERR_ARG, "bad sample arguments");
     if (shots == 0) return QD_OK;
-    int rc = compute_cdf(r);
-    if (rc) return rc;
-    double *u_dev = nullptr;
-    int64_t *o_dev = nullptr;
-    if (u_host && cudaMalloc(&u_dev, sizeof(double) * shots) != cudaSuccess) return fail(QD_ERR_OOM, "sample buffer");
-    if (cudaMalloc(&o_dev, sizeof(int64_t) * shots) != cudaSuccess) {
-        if (u_dev) cudaFree(u_dev);
-        return fail(QD_ERR_OOM, "sample buffer");
+    if (!r->samp && cudaMalloc(&r->samp, sizeof(double) * sample_doubles((uint64_t)r->N)) != cudaSuccess) {
+        cudaGetLastError();
+        r->samp = nullptr;
+        return fail(QD_ERR_OOM, "sampling prefix sums allocation failed");
     }
+    // draws and uniforms of up to kShotKeep bytes stay with the register; a
+    // larger call's are its own
+    const size_t need = (size_t)shots * (u_host ? 16 : 8);
+    void *buf = nullptr;
+    const bool keep = need <= kShotKeep;
+    if (keep && r->shot_cap >= need) {
+        buf = r->shot;
+    } else {
+        if (keep && r->shot) {
+            cudaFree(r->shot);
+            r->shot = nullptr;
+            r->shot_cap = 0;
+        }
+        const size_t bytes = keep ? std::max<size_t>(need, size_t(1) << 16) : need;
+        if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(QD_ERR_OOM, "sample buffer");
+        }
+        if (keep) {
+            r->shot = buf;
+            r->shot_cap = bytes;
+        }
+    }
+    int64_t *o_dev = static_cast<int64_t *>(buf);
+    double *u_dev = u_host ? reinterpret_cast<double *>(o_dev + shots) : nullptr;
     cudaError_t e = cudaSuccess;
     if (u_host) e = cudaMemcpyAsync(u_dev, u_host, sizeof(double) * shots, cudaMemcpyHostToDevice, r->stream);
-    if (e == cudaSuccess) e = sample(r->cdf, (uint64_t)r->N, u_dev, seed, shots, o_dev, r->sm_count, r->stream);
+    if (e == cudaSuccess)
+        e = sample(r->psi, r->prec, (uint64_t)r->N, r->samp, u_dev, seed, shots, o_dev, r->sm_count, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, o_dev, sizeof(int64_t) * shots, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
-    if (u_dev) cudaFree(u_dev);
-    cudaFree(o_dev);
+    if (!keep) cudaFree(buf);
     if (e != cudaSuccess) return cuda_fail(e, "sample");
     return QD_OK;
 }
