@@ -59,6 +59,8 @@ int cuda_fail(cudaError_t e, const char *where) {
 
 // ---------------------------------------------------------------- register
 
+constexpr int kDevWords = 8;
+
 struct qd_reg {
     int32_t n = 0;
     int32_t dims[QD_MAX_QUDITS] = {};
@@ -78,7 +80,7 @@ struct qd_reg {
     double *samp = nullptr;    // lazily allocated prefix sums of qd_sample
     void *shot = nullptr;      // device copies of a call's draws (and uniforms)
     size_t shot_cap = 0;       // bytes
-    int32_t *dev_err = nullptr;
+    int32_t *dev_err = nullptr;  // kDevWords words: the error word, and (from word 2) a kernel's tile queue
     int64_t tile_stride = -1;  // -1: process default
     int32_t fuse_kmax = 3;     // largest number of qudits of a fused block
     int32_t index64 = 0;       // 64-bit index kernels below 2^31 amplitudes too
@@ -150,6 +152,7 @@ cudaError_t launch_plan(const qd_reg *r, const GatePlan &g) {
         return diag_table_apply(r->psi, r->prec, (uint64_t)r->N, g.tab_div, g.tab_size, g.tab, r->sm_count, r->stream,
                                 g.wide);
     if (r->prec == QD_C64) return launch_gate_f32(g, r->psi, r->sm_count, r->stream);
+    if (tc64_takes(g)) return launch_dense_tc64(g, r->psi, r->sm_count, r->dev_err, r->stream);
     return launch_gate_f64(g, r->psi, r->sm_count, r->stream);
 }
 
@@ -672,8 +675,8 @@ int qd_create(const int32_t *dims, int32_t n, const int32_t *init_levels, int32_
         }
         r->owns = true;
     }
-    if (cudaMalloc(&r->dev_err, sizeof(int32_t)) != cudaSuccess ||
-        cudaMemsetAsync(r->dev_err, 0, sizeof(int32_t), r->stream) != cudaSuccess) {
+    if (cudaMalloc(&r->dev_err, kDevWords * sizeof(int32_t)) != cudaSuccess ||
+        cudaMemsetAsync(r->dev_err, 0, kDevWords * sizeof(int32_t), r->stream) != cudaSuccess) {
         cudaGetLastError();
         qd_destroy(r);
         return fail(QD_ERR_OOM, "error word allocation failed");

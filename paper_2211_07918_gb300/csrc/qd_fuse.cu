@@ -217,8 +217,19 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     double t_mem = 2.0 * touched * b / 5.0e12;
     if (table) t_mem += std::exp2((double)lf.f[0]) * 16.0 / 5.0e12;
     if (dense_table) t_mem += std::exp2((double)lf.f[11]) * 16.0 / 5.0e12;
+    // complex128 dense kernels: the CUDA cores take 4 D DFMA per amplitude; the
+    // tensor cores (qd_tc64.cu, measured on 3.4e7 amplitudes) 8.2 ps per
+    // amplitude up to D = 4, up to 16 9.6 ps at full rows of 8 or 16 slots and
+    // 1.3 times that with slots to spare, 15 ps above (one CTA per SM: its MMAs
+    // are not overlapped), and 5 us of setup
+    double t_c128 = touched * 4.0 * D / 0.5e12;
+    if (c128) {
+        const double Dp = std::ceil(D / 8.0) * 8.0;
+        const double t_tc = touched * (D <= 4.5 ? 8.2e-12 : D <= 16.5 ? 9.6e-12 * (1.0 + 0.65 * (Dp - D) / Dp) : 15.0e-12) + 1.0e-6;
+        t_c128 = std::min(t_c128, t_tc);
+    }
     double t_cmp = table ? touched * 40.0 / 2.0e13 : 0.0;  // index arithmetic per amplitude
-    if (dense_table) t_cmp = c128 ? touched * 4.0 * D / 0.5e12 : touched * (8.0 * D + 64.0) / 2.0e13;
+    if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : touched * (8.0 * D + 64.0) / 2.0e13;
     if (dense && !table && !dense_table) {
         if (!c128 && block) {
             // fused block on the tensor cores: 6 exact BF16 slice products of
@@ -227,9 +238,8 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
             const double Dp = D <= 32 ? std::ceil(D / 8.0) * 8.0 : std::ceil(D / 16.0) * 16.0;
             t_cmp = 2.0 * touched * b / (3.5e12 * D / Dp);
         } else {
-            // complex64 with hi+lo coefficients: 8 D FFMA per amplitude plus
-            // index work; complex128: 4 D DFMA per amplitude
-            t_cmp = c128 ? touched * 4.0 * D / 0.5e12 : touched * (8.0 * D + 24.0) / 2.0e13;
+            // complex64 with hi+lo coefficients: 8 D FFMA per amplitude plus index work
+            t_cmp = c128 ? t_c128 : touched * (8.0 * D + 24.0) / 2.0e13;
         }
     }
     return std::max(t_mem, t_cmp) + 4.0e-6;

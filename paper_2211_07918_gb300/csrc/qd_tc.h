@@ -23,4 +23,12 @@ int tc_smem_bytes(int Dp);
 // Launch one block (g.mode == Mode::Tensor) on a complex64 state.
 cudaError_t launch_block_tc(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
 
+// Dense gates and blocks of complex128 states (qd_tc64.cu): whether the kernel
+// takes a launch (direct geometry, matrix entries of ordinary size, for D < 4
+// enough amplitudes in the gate's slice), and the launch.  err: the
+// error word, followed by the queue words 2 and 3, zero between launches; the
+// launches that share it are ordered on one stream.
+bool tc64_takes(const GatePlan &g);
+cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
+
 }  // namespace qd
