@@ -28,6 +28,7 @@ SOURCES = [
     "qd_noalloc.cu",
     "qd_fuse.cu",
     "qd_tc.cu",
+    "qd_tc32.cu",
     "qd_tc64.cu",
     "qd_mlp.cu",
     "qd_batch.cu",

@@ -147,11 +147,16 @@ bool all_pow2(const qd_reg *r) {
 }
 
 cudaError_t launch_plan(const qd_reg *r, const GatePlan &g) {
-    if (g.mode == Mode::Tensor) return launch_block_tc(g, r->psi, r->sm_count, r->dev_err, r->stream);
+    if (g.mode == Mode::Tensor)
+        return g.tc_terms ? launch_block_tc(g, r->psi, r->sm_count, r->dev_err, r->stream)
+                          : launch_dense_tc32(g, r->psi, r->sm_count, r->dev_err, r->stream);
     if (g.mode == Mode::Table)
         return diag_table_apply(r->psi, r->prec, (uint64_t)r->N, g.tab_div, g.tab_size, g.tab, r->sm_count, r->stream,
                                 g.wide);
-    if (r->prec == QD_C64) return launch_gate_f32(g, r->psi, r->sm_count, r->stream);
+    if (r->prec == QD_C64) {
+        if (tc32_takes(g, false)) return launch_dense_tc32(g, r->psi, r->sm_count, r->dev_err, r->stream);
+        return launch_gate_f32(g, r->psi, r->sm_count, r->stream);
+    }
     if (tc64_takes(g)) return launch_dense_tc64(g, r->psi, r->sm_count, r->dev_err, r->stream);
     return launch_gate_f64(g, r->psi, r->sm_count, r->stream);
 }
@@ -955,7 +960,8 @@ int segments_for(const qd_reg *r, const std::vector<FuseGate> &fg, int plan_kind
 }
 
 // Tensor-core plan of one fused block (complex64): direct group geometry over
-// the block's qudits, no controls; the BF16 terms are packed into `terms`.
+// the block's qudits, no controls; the BF16 terms of a block for qd_tc.cu are
+// packed into `terms` (left empty for qd_tc32.cu).
 int plan_block_tc(const qd_reg *r, const FuseBlock &b, GatePlan &g, std::vector<uint16_t> &terms) {
     g = GatePlan{};
     g.mode = Mode::Tensor;
@@ -981,6 +987,13 @@ int plan_block_tc(const qd_reg *r, const FuseBlock &b, GatePlan &g, std::vector<
         g.off[j] = o;
     }
     g.alg_bytes = 2.0 * (double)r->N * (double)r->esize;
+    if (b.D <= 16) {  // qd_tc32.cu, its matrix in the launch's arguments; no terms
+        std::memcpy(g.U, b.M.data(), sizeof(double) * 2 * b.D * b.D);
+        g.mode = Mode::Direct;
+        const bool takes = tc32_takes(g, true);
+        g.mode = Mode::Tensor;
+        if (takes) return QD_OK;
+    }
     terms.resize(tc_terms_bytes(g.Dp) / 2);
     tc_pack_terms(b.M.data(), b.D, g.Dp, terms.data());
     return QD_OK;
@@ -1143,9 +1156,12 @@ int build_plan(qd_reg *r, const std::vector<FuseGate> &fg, const std::vector<con
             if ((int)b.qudits.size() > QD_MAX_TARGETS) {
                 rc = fail(QD_ERR_DIM, "fused block spans more than 6 qudits");
             } else if (b.D <= kTcMaxD && kinds[si] == kKernelBlockTc) {
-                tc_terms.emplace_back();
-                rc = plan_block_tc(r, b, g, tc_terms.back());
-                tc_index.push_back((int)p->gates.size());
+                std::vector<uint16_t> terms;
+                rc = plan_block_tc(r, b, g, terms);
+                if (!terms.empty()) {
+                    tc_terms.push_back(std::move(terms));
+                    tc_index.push_back((int)p->gates.size());
+                }
             } else {
                 rc = plan_block(r, b, g);
                 if (rc == QD_OK && g.D == 0) continue;

@@ -214,7 +214,8 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     // feature 11: log2 of the control-slice fraction, or (dense + table) of the table entries
     const double touched = dense_table ? (double)reg.N : (double)reg.N * std::exp2((double)lf.f[11]);
     const double b = c128 ? 16.0 : 8.0;
-    double t_mem = 2.0 * touched * b / 5.0e12;
+    // 5.4 TB/s: what the memory-bound dense kernels move on large registers
+    double t_mem = 2.0 * touched * b / (dense ? 5.4e12 : 5.0e12);
     if (table) t_mem += std::exp2((double)lf.f[0]) * 16.0 / 5.0e12;
     if (dense_table) t_mem += std::exp2((double)lf.f[11]) * 16.0 / 5.0e12;
     // complex128 dense kernels: the CUDA cores take 4 D DFMA per amplitude; the
@@ -229,17 +230,20 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
         t_c128 = std::min(t_c128, t_tc);
     }
     double t_cmp = table ? touched * 40.0 / 2.0e13 : 0.0;  // index arithmetic per amplitude
-    if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : touched * (8.0 * D + 64.0) / 2.0e13;
+    if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : D <= 4.5 ? 0.0 : touched * (8.0 * D + 64.0) / 2.0e13;
     if (dense && !table && !dense_table) {
         if (!c128 && block) {
-            // fused block on the tensor cores: 6 exact BF16 slice products of
-            // (2 Dp) x (2 Dp) per group; measured on GB300 the kernel moves
-            // about 3.5 TB/s at D = Dp, less in proportion to the padding
+            // fused block on the tensor cores: measured on GB300 it moves about
+            // 5.3 TB/s at D = Dp (4.95 above 32), less in proportion to the
+            // padding; up to D = 16 (qd_tc32.cu) 5.0 TB/s at full rows of 16 slots
             const double Dp = D <= 32 ? std::ceil(D / 8.0) * 8.0 : std::ceil(D / 16.0) * 16.0;
-            t_cmp = 2.0 * touched * b / (3.5e12 * D / Dp);
+            t_cmp = D < 16.5 ? touched * 5.1e-11 / D : 2.0 * touched * b / ((D <= 32 ? 5.3e12 : 4.95e12) * D / Dp);
         } else {
-            // complex64 with hi+lo coefficients: 8 D FFMA per amplitude plus index work
-            t_cmp = c128 ? t_c128 : touched * (8.0 * D + 24.0) / 2.0e13;
+            // complex64 with hi+lo coefficients: hidden under the memory pass up to
+            // D = 8, then 8 D FFMA per amplitude plus index work (packed at D = 9);
+            // from D = 10 to 16 the tensor cores (qd_tc32.cu) at rows of 16 slots
+            t_cmp = c128 ? t_c128 : D < 8.5 ? 0.0 : touched * (8.0 * D + 24.0) / (D < 9.5 ? 2.4e13 : 2.0e13);
+            if (!c128 && D > 9.5 && D < 16.5) t_cmp = std::min(t_cmp, touched * 5.1e-11 / D);
         }
     }
     return std::max(t_mem, t_cmp) + 4.0e-6;

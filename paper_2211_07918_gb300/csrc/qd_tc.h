@@ -31,4 +31,15 @@ cudaError_t launch_block_tc(const GatePlan &g, void *psi, int sm_count, int32_t 
 bool tc64_takes(const GatePlan &g);
 cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
 
+// Dense gates and blocks of complex64 states of kTcMinD to 16 states
+// (qd_tc32.cu): whether the kernel takes a launch (direct geometry, matrix
+// entries of ordinary size; for a single gate or a block priced on the CUDA
+// cores, the shapes at which it is the faster one), and the launch.
+bool tc32_takes(const GatePlan &g, bool block);
+cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
+
+// Whether the exponent field of every matrix row's largest entry lies in
+// [low, high] (rows of zeros aside).
+bool tc_matrix_ordinary(const GatePlan &g, int low, int high);
+
 }  // namespace qd

@@ -584,16 +584,7 @@ bool tc64_takes(const GatePlan &g) {
     const double amps = (double)g.R * g.D;
     if (g.D == 2 && amps < 300000) return false;
     if (g.D == 3 && amps < 180000) return false;
-    for (int i = 0; i < g.D; ++i) {
-        int top = 0;
-        for (int k = 0; k < 2 * g.D; ++k) {
-            uint64_t b;
-            std::memcpy(&b, &g.U[2 * i * g.D + k], 8);
-            top = std::max(top, (int)((b >> 52) & 0x7ff));
-        }
-        if (top && (top < kMatExLow || top > kMatExHigh)) return false;
-    }
-    return true;
+    return tc_matrix_ordinary(g, kMatExLow, kMatExHigh);
 }
 
 cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {

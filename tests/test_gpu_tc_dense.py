@@ -1,5 +1,5 @@
-"""Dense complex128 gates on the tensor cores: every dimension, slot layout,
-ragged tiles, controls and both index widths against extended precision."""
+"""Dense gates on the tensor cores in both precisions: every dimension, slot
+layout, ragged tiles, controls and both index widths against extended precision."""
 import math
 
 import numpy as np
@@ -9,6 +9,18 @@ from paper_2211_07918_gb300 import qudit as L
 from paper_2211_07918_gb300 import workloads as wl
 
 pytestmark = pytest.mark.gpu
+BOTH = [L.QD_C64, L.QD_C128]
+DTYPE = {L.QD_C64: np.complex64, L.QD_C128: np.complex128}
+
+
+def bound(prec, d):
+    """Largest error of a part of the result of a unitary gate, in units of the group's largest part.
+
+    complex128: 2 D products of parts off by at most half a last place of the largest, the matrix
+    entries likewise, one rounding of the result: below 4 D 2^-53.  complex64: parts off by 2^-26 of
+    the largest, sqrt(2 D) in sum, and four FP32 roundings of a result of at most sqrt(2 D):
+    below sqrt(2 D) 2^-22."""
+    return 4 * d * 2.0 ** -53 if prec == L.QD_C128 else math.sqrt(2 * d) * 2.0 ** -22
 
 
 def apply_ref(psi, dims, m, targets, controls=(), levels=()):
@@ -25,31 +37,31 @@ def apply_ref(psi, dims, m, targets, controls=(), levels=()):
     return t.ravel()
 
 
-def check(dims, targets, controls=(), levels=(), index64=0, seed=0, scale=1.0):
+def check(prec, dims, targets, controls=(), levels=(), index64=0, seed=0, scale=1.0):
     rng = np.random.default_rng(seed)
     n, d = math.prod(dims), math.prod(dims[q] for q in targets)
     psi = (rng.standard_normal(n) + 1j * rng.standard_normal(n)) * scale
     psi[rng.random(n) < 0.05] = 0
+    psi = psi.astype(DTYPE[prec])
     m = wl.haar_unitary(d, rng)
-    with L.Register(dims, None, L.QD_C128) as r:
+    with L.Register(dims, None, prec) as r:
         L.qd_set_tuning(r.h, L.QD_TUNE_INDEX64, index64)
         L.qd_set_amplitudes(r.h, psi)
         L.qd_apply(r.h, m, targets, controls, levels or None)
         L.qd_sync(r.h)
         got = r.amplitudes()
     want = apply_ref(psi, dims, m, targets, tuple(controls), tuple(levels))
-    # per part: 2 D products of parts off by at most half a last place of the largest, the matrix
-    # entries likewise, one rounding of the result: below 4 D 2^-53 of the largest part
     err = np.max(np.abs((got - want).astype(np.complex128)))
-    assert err <= 4 * d * 2.0 ** -53 * np.max(np.abs(psi)), (err, d)
+    assert err <= bound(prec, d) * np.max(np.abs(psi)), (err, d)
     if controls:  # amplitudes outside the control slice are untouched
         same = apply_ref(psi, dims, np.zeros((d, d)), targets, tuple(controls), tuple(levels)) != 0
         assert np.array_equal(got[same], psi[same])
 
 
+@pytest.mark.parametrize("prec", BOTH)
 @pytest.mark.parametrize("index64", [0, 1])
 @pytest.mark.parametrize("d", list(range(2, 33)))
-def test_every_dimension(d, index64):
+def test_every_dimension(d, index64, prec):
     # 1 qudit of d levels below, inside and above others; a group count that fills no tile evenly
     n_other = {2: 310000, 3: 190000}.get(d, 17000) // d // 7 + 1
     a = next(x for x in range(64, 1, -1) if n_other / x > 1)
@@ -57,22 +69,24 @@ def test_every_dimension(d, index64):
     c = max(2, -(-n_other // (a * b)))
     for dims, t in (([d, 7, a, b, c], 0), ([7, a, d, b, c], 2), ([7, c, a, b, d], 4)):
         assert math.prod(dims) >= {2: 300000, 3: 180000}.get(d, 16384)
-        check(dims, [t], index64=index64, seed=d)
+        check(prec, dims, [t], index64=index64, seed=d)
 
 
+@pytest.mark.parametrize("prec", BOTH)
 @pytest.mark.parametrize("dims,targets,controls,levels", [
     ([2] * 17, [3, 9], [], []), ([2] * 17, [0, 1, 2], [], []), ([2] * 18, [16, 2, 7, 5], [4], [0]),
     ([3] * 11, [4, 0], [], []), ([3] * 11, [0, 1, 2], [], []), ([3] * 14, [7], [0, 3], [2, 1]),
     ([4, 3, 2] * 4, [0, 3], [1], [1]), ([5, 2, 4, 3, 4, 5, 3, 4, 4], [5, 0], [], []),
     ([2, 64, 9, 16], [0, 3], [], []), ([3] * 12 + [2, 2], [13], [12], [1])], ids=str)
-def test_geometries(dims, targets, controls, levels):
-    check(dims, targets, controls, levels, seed=3)
-    check(dims, targets, controls, levels, seed=4, scale=1e-90)
+def test_geometries(dims, targets, controls, levels, prec):
+    check(prec, dims, targets, controls, levels, seed=3)
+    check(prec, dims, targets, controls, levels, seed=4, scale=1e-90 if prec == L.QD_C128 else 1e-15)
 
 
+@pytest.mark.parametrize("prec", BOTH)
 @pytest.mark.parametrize("dims,target", [([2] * 19, 4), ([3] * 11 + [2], 2), ([5] * 7, 1), ([20, 4, 5, 5, 9], 0), ([31, 9, 8, 8], 0)],
                          ids=str)
-def test_groups_outside_the_integers_range(dims, target):
+def test_groups_outside_the_integers_range(dims, target, prec):
     """Infinities, NaN, and groups of extremely small or large amplitudes go through FP64; their
     neighbours are not affected, and a group keeps its own scale."""
     rng = np.random.default_rng(5)
@@ -81,14 +95,15 @@ def test_groups_outside_the_integers_range(dims, target):
     s = math.prod(dims[:target])
     group = np.arange(n) // (s * d) * s + np.arange(n) % s
     kind = group % 97
-    psi[kind == 1] *= 1e-250
-    psi[kind == 2] *= 1e+290
+    psi[kind == 1] *= 1e-250 if prec == L.QD_C128 else 1e-34
+    psi[kind == 2] *= 1e+290 if prec == L.QD_C128 else 1e+34
     psi[kind == 3] *= 1e-12
     psi[kind == 4] = 0
     psi[(kind == 5) & (np.arange(n) // s % d == 1)] = np.inf
     psi[(kind == 6) & (np.arange(n) // s % d == 0)] = complex(np.nan, 1)
+    psi = psi.astype(DTYPE[prec])
     m = wl.haar_unitary(d, rng)
-    with L.Register(dims, None, L.QD_C128) as r:
+    with L.Register(dims, None, prec) as r:
         L.qd_set_amplitudes(r.h, psi)
         L.qd_apply(r.h, m, [target])
         L.qd_sync(r.h)
@@ -98,29 +113,32 @@ def test_groups_outside_the_integers_range(dims, target):
     fine = (kind != 5) & (kind != 6)
     largest = np.zeros(group.max() + 1)
     np.maximum.at(largest, group[fine], np.abs(psi[fine]))
-    assert np.all(np.abs((got - want)[fine].astype(np.complex128)) <= 4 * d * 2.0 ** -53 * largest[group[fine]])
+    floor = 0 if prec == L.QD_C128 else 2.0 ** -148  # results below the normal numbers
+    assert np.all(np.abs((got[fine] - want[fine]).astype(np.complex128)) <= bound(prec, d) * largest[group[fine]] + floor)
     assert not np.any(np.isfinite(got.real[~fine]) & np.isfinite(got.imag[~fine]))
 
 
+@pytest.mark.parametrize("prec", BOTH)
 @pytest.mark.parametrize("d", [2, 3, 4, 7, 9, 16, 20, 27, 32])
-def test_leading_digits_at_their_limits(d):
+def test_leading_digits_at_their_limits(d, prec):
     """Amplitudes and matrix entries just below, at and above powers of two."""
     rng = np.random.default_rng(d)
-    n_other = 20000 // d // 8 + 1
-    dims = [4, d, 2, 64, n_other // 64 + 2]
+    n_other = {2: 300000, 3: 180000}.get(d, 20000) // d // 8 + 1
+    dims = [4, d, 2, 64, min(64, n_other // 64 + 2), n_other // 4096 + 2]
     near = np.array([s * (1 + t * 2.0 ** -k) for s in (1, -1) for t in (1, -1, 0) for k in range(1, 54)])
     n = math.prod(dims)
-    psi = rng.choice(near, n) + 1j * rng.choice(near, n)
+    psi = (rng.choice(near, n) + 1j * rng.choice(near, n)).astype(DTYPE[prec])
     m = rng.choice(near, (d, d)) + 1j * rng.choice(near, (d, d))
-    with L.Register(dims, None, L.QD_C128) as r:
+    with L.Register(dims, None, prec) as r:
         L.qd_set_amplitudes(r.h, psi)
         L.qd_apply(r.h, m, [1])
         L.qd_sync(r.h)
         got = r.amplitudes()
     # matrix rows of largest part up to 1.5, amplitudes up to 1.5, 2 D products of parts, each side
-    # off by half a last place of the largest: 2 D (2 2^-53 1.5 1.5) and one rounding
+    # off by half a last place of the largest: 2 D (2 2^-53 1.5 1.5) and one rounding; complex64:
+    # 2 D 2.25 (2^-26 and four roundings of 2^-24)
     err = np.max(np.abs((got - apply_ref(psi, dims, m, [1])).astype(np.complex128)))
-    assert err <= 12 * d * 2.0 ** -53, err
+    assert err <= (12 * d * 2.0 ** -53 if prec == L.QD_C128 else 6 * d * 2.0 ** -23), err
 
 
 @pytest.mark.parametrize("index64", [0, 1])
