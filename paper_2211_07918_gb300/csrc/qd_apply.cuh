@@ -23,6 +23,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "qd_launch.cuh"
 #include "qd_plan.h"
 
 namespace qd {
@@ -194,6 +195,8 @@ __host__ __device__ constexpr int direct_min_blocks() {
 
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256, (direct_min_blocks<T, MD, true>())) k_dense_direct(const __grid_constant__ DenseDirectArgs<T, I, MD> a) {
+    chain_release();
+    chain_wait();
     constexpr int UN = direct_unroll<T, I, MD>();
     const int D = EX ? MD : a.D;
     const I step = (I)gridDim.x * blockDim.x;
@@ -294,6 +297,8 @@ __global__ void __launch_bounds__(256, (direct_min_blocks<T, MD, true>())) k_den
 
 template <typename T, typename I, int MD>
 __global__ void __launch_bounds__(256, (direct_min_blocks<T, MD, false>())) k_mono_direct(const __grid_constant__ MonoDirectArgs<T, I, MD> a) {
+    chain_release();
+    chain_wait();
     constexpr int UN = mono_unroll<T, I, MD>();
     const I step = (I)gridDim.x * blockDim.x;
     for (I r0 = (I)blockIdx.x * blockDim.x + threadIdx.x; r0 < a.R; r0 += UN * step) {
@@ -373,6 +378,8 @@ __host__ __device__ constexpr int table_min_blocks() {
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256, (table_min_blocks<T, I, MD>()))
     k_dense_table(const __grid_constant__ DenseTableArgs<T, I, MD> a) {
+    chain_release();
+    chain_wait();
     constexpr int UN = MD <= 4 ? 2 : 1;
     constexpr int TB = MD <= 4 ? MD : 2;  // outputs whose entries are loaded together
     using Entry = typename TabEntry<T>::type;
@@ -510,6 +517,8 @@ __device__ __forceinline__ void tile_store(const TileGeo<I> &t, v2<T> *psi, uint
 
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256) k_dense_tile(const __grid_constant__ DenseTileArgs<T, I, MD> a) {
+    chain_release();
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     const TileGeo<I> &t = a.t;
     const int D = EX ? MD : a.D;
@@ -549,6 +558,8 @@ __global__ void __launch_bounds__(256) k_dense_tile(const __grid_constant__ Dens
 
 template <typename T, typename I, int MD>
 __global__ void __launch_bounds__(256) k_mono_tile(const __grid_constant__ MonoTileArgs<T, I, MD> a) {
+    chain_release();
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     const TileGeo<I> &t = a.t;
     I *cbase = reinterpret_cast<I *>(smraw);
@@ -708,8 +719,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
         auto fn = k_dense_direct<T, I, MD, EX>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        fn<<<grid, kBlock, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(fn, grid, kBlock, 0, s, a);
     }
     DenseTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -726,8 +736,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, kBlock, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kBlock, smem, s, a);
 }
 
 // A permutation with phases whose moved members are few (a fused Toffoli
@@ -766,8 +775,7 @@ cudaError_t launch_mono_compact(const GatePlan &g, void *psi, int sm_count, cuda
     auto fn = k_mono_direct<T, I, MD>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, kBlock, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kBlock, 0, s, a);
 }
 
 template <typename T, typename I, int MD>
@@ -789,8 +797,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
         auto fn = k_mono_direct<T, I, MD>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        fn<<<grid, kBlock, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(fn, grid, kBlock, 0, s, a);
     }
     MonoTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -810,8 +817,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, kBlock, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kBlock, smem, s, a);
 }
 
 template <typename T, typename I, int MD, bool EX>
@@ -845,8 +851,7 @@ cudaError_t launch_dense_table(const GatePlan &g, void *psi, int sm_count, cudaS
     auto fn = k_dense_table<T, I, MD, EX>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, kBlock, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kBlock, 0, s, a);
 }
 
 template <typename T, typename I>

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "qd_diag.h"
+#include "qd_launch.cuh"
 
 namespace qd {
 
@@ -70,6 +71,8 @@ __global__ void __launch_bounds__(kDiagBlock) k_diag_apply_f32(float2 *__restric
                                                                typename DivOf<I>::type divA,
                                                                typename DivOf<I>::type divT,
                                                                const float4 *__restrict__ tab) {
+    chain_release();
+    chain_wait();
     const I step = (I)gridDim.x * blockDim.x * 4;
     for (I i0 = diag_chunk0<I>(); i0 < N; i0 += step) {
         float2 v[4];
@@ -103,6 +106,8 @@ __global__ void __launch_bounds__(kDiagBlock) k_diag_apply_f64(double2 *__restri
                                                                typename DivOf<I>::type divA,
                                                                typename DivOf<I>::type divT,
                                                                const double2 *__restrict__ tab) {
+    chain_release();
+    chain_wait();
     const I step = (I)gridDim.x * blockDim.x * 4;
     for (I i0 = diag_chunk0<I>(); i0 < N; i0 += step) {
         double2 v[4], t[4];
@@ -149,24 +154,25 @@ cudaError_t diag_table_apply(void *psi, int prec, uint64_t N, uint64_t s_qa, uin
                              int sm_count, cudaStream_t s, bool wide) {
     const int grid = grid_for(N, 4, sm_count);
     if (grid <= 0) return cudaSuccess;
+    cudaError_t e;
     if (N < (uint64_t(1) << 31) && !wide) {
         const FastDiv32 a = make_fastdiv32((uint32_t)s_qa), t = make_fastdiv32((uint32_t)TS);
         if (prec == 1)
-            k_diag_apply_f32<uint32_t><<<grid, kDiagBlock, 0, s>>>(static_cast<float2 *>(psi), (uint32_t)N, a, t,
+            e = launch_chained(k_diag_apply_f32<uint32_t>, grid, kDiagBlock, 0, s, static_cast<float2 *>(psi), (uint32_t)N, a, t,
                                                                    static_cast<const float4 *>(tab));
         else
-            k_diag_apply_f64<uint32_t><<<grid, kDiagBlock, 0, s>>>(static_cast<double2 *>(psi), (uint32_t)N, a, t,
+            e = launch_chained(k_diag_apply_f64<uint32_t>, grid, kDiagBlock, 0, s, static_cast<double2 *>(psi), (uint32_t)N, a, t,
                                                                    static_cast<const double2 *>(tab));
     } else {
         const FastDiv64 a = make_fastdiv64(s_qa), t = make_fastdiv64(TS);
         if (prec == 1)
-            k_diag_apply_f32<uint64_t><<<grid, kDiagBlock, 0, s>>>(static_cast<float2 *>(psi), N, a, t,
+            e = launch_chained(k_diag_apply_f32<uint64_t>, grid, kDiagBlock, 0, s, static_cast<float2 *>(psi), N, a, t,
                                                                    static_cast<const float4 *>(tab));
         else
-            k_diag_apply_f64<uint64_t><<<grid, kDiagBlock, 0, s>>>(static_cast<double2 *>(psi), N, a, t,
+            e = launch_chained(k_diag_apply_f64<uint64_t>, grid, kDiagBlock, 0, s, static_cast<double2 *>(psi), N, a, t,
                                                                    static_cast<const double2 *>(tab));
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace qd

@@ -10,6 +10,7 @@
 
 #include "qd_common.cuh"
 #include "qd_fixed.cuh"
+#include "qd_launch.cuh"
 #include "qd_reduce.h"
 
 namespace qd {
@@ -36,6 +37,8 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
 // psi = 0 except psi[idx] = 1.
 template <typename T>
 __global__ void k_init(v2<T> *psi, uint64_t N, uint64_t idx) {
+    chain_release();
+    chain_wait();
     const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += step)
         psi[i] = mk<T>(i == idx ? T(1) : T(0), T(0));
@@ -545,9 +548,8 @@ int grid_for(uint64_t n, int block, int sm_count, int per_sm) {
 
 cudaError_t init_basis(void *psi, int prec, uint64_t N, uint64_t idx, int sm_count, cudaStream_t s) {
     const int g = grid_for(N, 256, sm_count, 8);
-    if (prec == 1) k_init<float><<<g, 256, 0, s>>>(static_cast<float2 *>(psi), N, idx);
-    else k_init<double><<<g, 256, 0, s>>>(static_cast<double2 *>(psi), N, idx);
-    return cudaGetLastError();
+    if (prec == 1) return launch_chained(k_init<float>, g, 256, 0, s, static_cast<float2 *>(psi), N, idx);
+    return launch_chained(k_init<double>, g, 256, 0, s, static_cast<double2 *>(psi), N, idx);
 }
 
 // the resident blocks of the sums (256 threads of at most 48 registers)

@@ -69,6 +69,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "qd_launch.cuh"
 #include "qd_plan.h"
 #include "qd_tc.h"
 #include "qd_umma.cuh"
@@ -261,6 +262,9 @@ __global__ void __launch_bounds__(TcCfg<MAXD>::THREADS, 1) k_block_tc(const __gr
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+
+    chain_release();  // this CTA has its TMEM
+    chain_wait();
 
     const I ntiles = (a.R + kTcRows - 1) / kTcRows;
     const I nlocal = (I)blockIdx.x < ntiles ? (ntiles - (I)blockIdx.x + (I)gridDim.x - 1) / (I)gridDim.x : 0;
@@ -622,8 +626,7 @@ static cudaError_t launch_tc_im(const GatePlan &g, void *psi, int sm_count, int3
     const uint64_t cap = (uint64_t)sm_count * occ;
     const int grid = (int)(tiles < cap ? tiles : cap);
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, C::THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, C::THREADS, (size_t)smem, s, a);
 }
 
 template <typename I>

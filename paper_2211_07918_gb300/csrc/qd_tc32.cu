@@ -38,6 +38,7 @@
 
 #include <cuda_runtime.h>
 
+#include "qd_launch.cuh"
 #include "qd_plan.h"
 #include "qd_tc.h"
 #include "qd_umma.cuh"
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_dense_tc32(const __grid_co
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    chain_release();  // this CTA has its TMEM
     // digits of the real embedding, rows 2i: (ur, -ui), 2i + 1: (ui, ur)
     for (int e = tid; e < a.D * a.D; e += kThreads) {
         const int i = e / a.D, j = e - i * a.D;
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_dense_tc32(const __grid_co
         }
     };
 
+    chain_wait();
     bool dead = false, issued = false;
     uint32_t par = 0;
     I t = (I)blockIdx.x;
@@ -375,8 +378,7 @@ cudaError_t launch_fn(const Tc32Args<I> &a, int sm_count, cudaStream_t s) {
     const uint64_t tiles = ((uint64_t)a.R + kRows - 1) / kRows;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * kPerSm);
     if (grid <= 0) return cudaSuccess;
-    fn<<<grid, kThreads, kData, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kThreads, kData, s, a);
 }
 
 // Exponent field of the matrix' largest part.
