@@ -719,7 +719,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
         auto fn = k_dense_direct<T, I, MD, EX>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        return launch_chained(fn, grid, kBlock, 0, s, a);
+        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
     }
     DenseTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -736,7 +736,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, smem, s, a);
+    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), a);
 }
 
 // A permutation with phases whose moved members are few (a fused Toffoli
@@ -775,7 +775,7 @@ cudaError_t launch_mono_compact(const GatePlan &g, void *psi, int sm_count, cuda
     auto fn = k_mono_direct<T, I, MD>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, 0, s, a);
+    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
 }
 
 template <typename T, typename I, int MD>
@@ -797,7 +797,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
         auto fn = k_mono_direct<T, I, MD>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        return launch_chained(fn, grid, kBlock, 0, s, a);
+        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
     }
     MonoTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -817,7 +817,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, smem, s, a);
+    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), a);
 }
 
 template <typename T, typename I, int MD, bool EX>
@@ -851,7 +851,7 @@ cudaError_t launch_dense_table(const GatePlan &g, void *psi, int sm_count, cudaS
     auto fn = k_dense_table<T, I, MD, EX>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, 0, s, a);
+    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
 }
 
 template <typename T, typename I>

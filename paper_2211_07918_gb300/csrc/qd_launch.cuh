@@ -9,20 +9,27 @@
 // come onto the SMs: at its start, or, if it allocates TMEM, after that (the
 // next kernel's blocks must not take TMEM that this kernel's still need).
 // Kernels and copies launched without the attribute wait for completion as
-// usual.  Measured: 500 gates on 4.8e6 complex64 amplitudes in L2 3747 -> 3567
+// usual.  Only states that fit the L2 cache are chained: on large
+// ones the latency is nothing against the pass (direct gate calls on 4.3e8
+// amplitudes 10.80 ms chained, 10.62 not).  Measured: 500 gates on 4.8e6 complex64 amplitudes in L2 3747 -> 3567
 // us; 40 gates on 324 complex128 amplitudes, planned, run and read, 497 -> 398 us.
 #pragma once
-#include <cuda_runtime.h>
-
+#include <cstdint>
 #include <utility>
+
+#include <cuda_runtime.h>
 
 namespace qd {
 
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+constexpr uint64_t kChainBytes = uint64_t(128) << 20;
+
+// state_bytes: the size of the state the kernel works on.
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t s, A &&...args) {
+inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t s, uint64_t state_bytes,
+                                  A &&...args) {
     cudaLaunchConfig_t c{};
     c.gridDim = dim3((unsigned)grid);
     c.blockDim = dim3((unsigned)block);
@@ -32,7 +39,7 @@ inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t 
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
-    c.numAttrs = s ? 1 : 0;  // the legacy default stream orders whole kernels
+    c.numAttrs = s && state_bytes <= kChainBytes ? 1 : 0;  // (the legacy default stream orders whole kernels)
     return cudaLaunchKernelEx(&c, fn, std::forward<A>(args)...);
 }
 

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_dense_tc32(const __grid_co
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    chain_release();  // this CTA has its TMEM
+    chain_wait();  // (no chain_release(): with it the compiler spilled the prefetched amplitudes, 217 -> 250 us)
     // digits of the real embedding, rows 2i: (ur, -ui), 2i + 1: (ui, ur)
     for (int e = tid; e < a.D * a.D; e += kThreads) {
         const int i = e / a.D, j = e - i * a.D;
@@ -251,7 +251,6 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_dense_tc32(const __grid_co
         }
     };
 
-    chain_wait();
     bool dead = false, issued = false;
     uint32_t par = 0;
     I t = (I)blockIdx.x;
@@ -368,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_dense_tc32(const __grid_co
 }
 
 template <typename I, bool PAIRS>
-cudaError_t launch_fn(const Tc32Args<I> &a, int sm_count, cudaStream_t s) {
+cudaError_t launch_fn(const Tc32Args<I> &a, uint64_t N, int sm_count, cudaStream_t s) {
     auto fn = k_dense_tc32<I, PAIRS>;
     // (the default split of the L1 memory may hold fewer CTAs)
     cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kData);
@@ -378,7 +377,7 @@ cudaError_t launch_fn(const Tc32Args<I> &a, int sm_count, cudaStream_t s) {
     const uint64_t tiles = ((uint64_t)a.R + kRows - 1) / kRows;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * kPerSm);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kThreads, kData, s, a);
+    return launch_chained(fn, grid, kThreads, kData, s, 8 * N, a);
 }
 
 // Exponent field of the matrix' largest part.
@@ -420,7 +419,7 @@ cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, c
             const double *u = &g.U[2 * (perm[i] * g.D + perm[j])];
             a.U[i * g.D + j] = make_double2(u[0], u[1]);
         }
-    return pairs ? launch_fn<I, true>(a, sm_count, s) : launch_fn<I, false>(a, sm_count, s);
+    return pairs ? launch_fn<I, true>(a, g.N, sm_count, s) : launch_fn<I, false>(a, g.N, sm_count, s);
 }
 
 }  // namespace

@@ -326,6 +326,7 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     chain_release();  // this CTA has its TMEM
+    chain_wait();
     // scale of the matrix row (a zero row: any)
     if (mine)
         atomicMax(&mat_ex[mi], (int)max((uint32_t)__double2hiint(u.x) & 0x7fffffffu, (uint32_t)__double2hiint(u.y) & 0x7fffffffu));
@@ -369,7 +370,6 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
         }
     };
 
-    chain_wait();
     bool dead = false, issued = false;
     uint32_t par = 0, coming = 0;
     if (QUEUE && tid == 0) coming = gridDim.x + atomicAdd(a.queue, 1u);  // the tile after this one
@@ -551,7 +551,7 @@ cudaError_t launch_tab(const GatePlan &g, void *psi, int sm_count, int32_t *err,
     const uint64_t tiles = (g.R + C::PER_TILE - 1) / C::PER_TILE;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * C::PER_SM);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, C::THREADS, C::DATA, s, a, tb);
+    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, a, tb);
 }
 
 template <typename I, int NP, int GD>
