@@ -64,8 +64,9 @@ __device__ __forceinline__ void load_pair(const v2<T> *__restrict__ psi, uint64_
 }
 
 // Amplitudes per thread and iteration of the sums below: the loads in flight
-// (64 bytes a thread for complex64, 128 for complex128) and the group whose
-// squares are added on the integer units (qd_fixed.cuh).
+// (64 bytes a thread) and the group whose squares are added on the integer
+// units (qd_fixed.cuh).  (Two of ten complex64 amplitudes on the FP64 pipe
+// beside them made it the limit: the norm of 3.4e8 took 644 us, not 508.)
 template <typename T> constexpr int kSumGroup = sizeof(T) == 4 ? 8 : 4;
 
 // Per-block partial sums of |psi_i|^2 over the whole state.  Bound by the
@@ -173,20 +174,23 @@ __global__ void k_sum_partials(const double *__restrict__ part, int nb, double *
 // (qd_fixed.cuh), two FP64 additions per group.  In FP64 the conversions and
 // products are eight operations of its pipe per complex64 pair.  3.4e8
 // amplitudes: complex64 pairs 5098 -> 1850 us, complex64 with complex128
-// 3882 -> 2014 us (4.05 TB/s), complex128 pairs 2416 -> 2390 us; the ALU pipe
-// is the limit now (139 instructions per mixed pair).
+// 3882 -> 1806 us (4.5 TB/s; 2014 without the FP64 pipe's share), complex128
+// pairs 2416 -> 2056 us (5.3 TB/s; 2390); the ALU pipe is the limit now (139
+// instructions per mixed pair).
 template <typename TA, typename TB>
 __global__ void __launch_bounds__(kRedBlock) k_overlap_partial(const v2<TA> *__restrict__ a, const v2<TB> *__restrict__ b,
                                                                uint64_t N, double *__restrict__ part) {
     __shared__ double sh[32];
-    constexpr int G = 4;
-    const uint64_t tile = (uint64_t)G * kRedBlock;
+    // a group on the integer units and, with a complex128 state (no or half the
+    // conversions), two pairs on the FP64 pipe beside it
+    constexpr int G = 4, F = sizeof(TA) + sizeof(TB) > 8 ? 2 : 0;
+    const uint64_t tile = (uint64_t)(G + F) * kRedBlock;
     double re = 0.0, im = 0.0;
     for (uint64_t t = (uint64_t)blockIdx.x * tile; t < N; t += (uint64_t)gridDim.x * tile) {
-        v2<TA> x[G];
-        v2<TB> y[G];
+        v2<TA> x[G + F];
+        v2<TB> y[G + F];
 #pragma unroll
-        for (int k = 0; k < G / 2; ++k) {
+        for (int k = 0; k < (G + F) / 2; ++k) {
             const uint64_t i = t + 2 * (k * kRedBlock + threadIdx.x);
             load_pair<TA>(a, i, N, x + 2 * k);
             load_pair<TB>(b, i, N, y + 2 * k);
@@ -195,6 +199,12 @@ __global__ void __launch_bounds__(kRedBlock) k_overlap_partial(const v2<TA> *__r
         group_overlap<TA, TB, G>(x, y, gr, gi);
         re += gr;
         im += gi;
+#pragma unroll
+        for (int k = G; k < G + F; ++k) {
+            const double xr = (double)x[k].x, xi = (double)x[k].y, yr = (double)y[k].x, yi = (double)y[k].y;
+            re = fma(xr, yr, fma(xi, yi, re));
+            im = fma(xr, yi, fma(-xi, yr, im));
+        }
     }
     re = block_sum(re, sh);
     im = block_sum(im, sh);
