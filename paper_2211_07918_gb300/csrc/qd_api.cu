@@ -78,8 +78,8 @@ struct qd_reg {
     double *cdf = nullptr;  // lazily allocated N doubles
     double *cdf_chunks = nullptr;
     double *samp = nullptr;    // lazily allocated prefix sums of qd_sample
-    void *shot = nullptr;      // device copies of a call's draws (and uniforms)
-    size_t shot_cap = 0;       // bytes
+    void *scratch = nullptr;   // device buffers of one readout call (draws, kets), kept up to kScratchKeep
+    size_t scratch_cap = 0;    // bytes
     int32_t *dev_err = nullptr;  // kDevWords words: the error word, and (from word 2) a kernel's tile queue
     int64_t tile_stride = -1;  // -1: process default
     int32_t fuse_kmax = 3;     // largest number of qudits of a fused block
@@ -309,7 +309,7 @@ int plan_gate(const qd_reg *r, const double *M, const Acting &a, bool diag_only,
     // matrix / classification
     if (force_dense) {  // the dense kernels, whatever the matrix (a dense part with a table epilogue)
         g.kind = Kind::Dense;
-        std::memcpy(g.U, M, sizeof(double) * 2 * D * D);
+        g.U.assign(M, M + 2 * D * D);
     } else if (diag_only) {
         for (int i = 0; i < D; ++i) {
             g.src[i] = i;
@@ -327,7 +327,7 @@ int plan_gate(const qd_reg *r, const double *M, const Acting &a, bool diag_only,
         g.kind = Kind::Mono;
     } else {
         g.kind = Kind::Dense;
-        std::memcpy(g.U, M, sizeof(double) * 2 * D * D);
+        g.U.assign(M, M + 2 * D * D);
     }
     if (g.kind == Kind::Mono && g.active == 0) {
         *noop = true;
@@ -573,6 +573,33 @@ int ensure_red(qd_reg *r, size_t doubles) {
     return QD_OK;
 }
 
+// Device scratch of one synchronous readout call: the register's own up to
+// kScratchKeep bytes (an allocation and its release cost more than a small
+// readout), else an allocation that the caller frees (*keep is false).  Null
+// when there is no memory.
+constexpr size_t kScratchKeep = size_t(1) << 24;
+
+void *reg_scratch(qd_reg *r, size_t need, bool *keep) {
+    *keep = need <= kScratchKeep;
+    if (*keep && r->scratch_cap >= need) return r->scratch;
+    if (*keep && r->scratch) {
+        cudaFree(r->scratch);
+        r->scratch = nullptr;
+        r->scratch_cap = 0;
+    }
+    void *buf = nullptr;
+    const size_t bytes = *keep ? std::max<size_t>(need, size_t(1) << 16) : need;
+    if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (*keep) {
+        r->scratch = buf;
+        r->scratch_cap = bytes;
+    }
+    return buf;
+}
+
 int ensure_cdf(qd_reg *r) {
     if (r->cdf) return QD_OK;
     const size_t nch = cdf_chunks((uint64_t)r->N) + 1;
@@ -709,7 +736,7 @@ int qd_destroy(qd_reg *r) {
     if (r->cdf) cudaFree(r->cdf);
     if (r->cdf_chunks) cudaFree(r->cdf_chunks);
     if (r->samp) cudaFree(r->samp);
-    if (r->shot) cudaFree(r->shot);
+    if (r->scratch) cudaFree(r->scratch);
     if (r->dev_err) cudaFree(r->dev_err);
     delete r;
     return QD_OK;
@@ -988,7 +1015,7 @@ int plan_block_tc(const qd_reg *r, const FuseBlock &b, GatePlan &g, std::vector<
     }
     g.alg_bytes = 2.0 * (double)r->N * (double)r->esize;
     if (b.D <= 16) {  // qd_tc32.cu, its matrix in the launch's arguments; no terms
-        std::memcpy(g.U, b.M.data(), sizeof(double) * 2 * b.D * b.D);
+        g.U = b.M;
         g.mode = Mode::Direct;
         const bool takes = tc32_takes(g, true);
         g.mode = Mode::Tensor;
@@ -1585,8 +1612,6 @@ int qd_cdf(qd_reg *r, double *out, int32_t where) {
     return QD_OK;
 }
 
-constexpr size_t kShotKeep = size_t(1) << 24;  // 1 to 2 million shots
-
 static int sample_impl(qd_reg *r, const double *u_host, uint64_t seed, int64_t shots, int64_t *out) {
     if (int rc = reg_ok(r)) return rc;
     if (!out || shots < 0) return fail(QD_ERR_ARG, "bad sample arguments");
@@ -1596,29 +1621,9 @@ static int sample_impl(qd_reg *r, const double *u_host, uint64_t seed, int64_t s
         r->samp = nullptr;
         return fail(QD_ERR_OOM, "sampling prefix sums allocation failed");
     }
-    // draws and uniforms of up to kShotKeep bytes stay with the register; a
-    // larger call's are its own
-    const size_t need = (size_t)shots * (u_host ? 16 : 8);
-    void *buf = nullptr;
-    const bool keep = need <= kShotKeep;
-    if (keep && r->shot_cap >= need) {
-        buf = r->shot;
-    } else {
-        if (keep && r->shot) {
-            cudaFree(r->shot);
-            r->shot = nullptr;
-            r->shot_cap = 0;
-        }
-        const size_t bytes = keep ? std::max<size_t>(need, size_t(1) << 16) : need;
-        if (cudaMalloc(&buf, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(QD_ERR_OOM, "sample buffer");
-        }
-        if (keep) {
-            r->shot = buf;
-            r->shot_cap = bytes;
-        }
-    }
+    bool keep = false;
+    void *buf = reg_scratch(r, (size_t)shots * (u_host ? 16 : 8), &keep);
+    if (!buf) return fail(QD_ERR_OOM, "sample buffer");
     int64_t *o_dev = static_cast<int64_t *>(buf);
     double *u_dev = u_host ? reinterpret_cast<double *>(o_dev + shots) : nullptr;
     cudaError_t e = cudaSuccess;
@@ -1667,30 +1672,43 @@ int qd_ket_list(qd_reg *r, int32_t method, double threshold, int64_t cap, int64_
     if (!(threshold >= 0.0)) return fail(QD_ERR_ARG, "threshold must be >= 0");
     const uint64_t nch = ket_chunks((uint64_t)r->N);
     const size_t per = method == QD_OUT_AMPLITUDE ? 2 : 1;
-    int64_t *counts = nullptr, *idx_dev = nullptr;
-    double *val_dev = nullptr;
+    // one block: counts, offsets (the last one is the total), indices, values
+    bool keep = false;
+    cap = std::min(cap, r->N);  // there are no more
+    const size_t head = 2 * (size_t)nch, words = head + 1 + (size_t)cap * (1 + per);
+    int64_t *counts = static_cast<int64_t *>(reg_scratch(r, 8 * words, &keep));
+    if (!counts) return fail(QD_ERR_OOM, "ket buffers");
+    int64_t *idx_dev = counts + head + 1;
+    double *val_dev = reinterpret_cast<double *>(idx_dev + cap);
     int rc = QD_OK;
-    if (cudaMalloc(&counts, sizeof(int64_t) * (2 * nch + 1)) != cudaSuccess) return fail(QD_ERR_OOM, "ket scratch");
-    if (cap > 0 && (cudaMalloc(&idx_dev, sizeof(int64_t) * cap) != cudaSuccess ||
-                    cudaMalloc(&val_dev, sizeof(double) * per * cap) != cudaSuccess))
-        rc = fail(QD_ERR_OOM, "ket output buffers");
     int64_t total = 0;
-    if (rc == QD_OK) {
-        int64_t *offsets = counts + nch;
-        cudaError_t e = ket_select(r->psi, r->prec, (uint64_t)r->N, threshold, method == QD_OUT_AMPLITUDE ? 0 : 1,
-                                   cap, counts, offsets, idx_dev, val_dev, r->sm_count, r->stream);
+    cudaError_t e = ket_select(r->psi, r->prec, (uint64_t)r->N, threshold, method == QD_OUT_AMPLITUDE ? 0 : 1, cap,
+                               counts, counts + nch, idx_dev, val_dev, r->sm_count, r->stream);
+    constexpr size_t kOneCopy = 8192;  // a short answer comes back in one piece
+    if (words - head <= kOneCopy) {
+        std::vector<int64_t> h(words - head);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&total, offsets + nch, sizeof(int64_t), cudaMemcpyDeviceToHost, r->stream);
+            e = cudaMemcpyAsync(h.data(), counts + head, 8 * h.size(), cudaMemcpyDeviceToHost, r->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
-        const int64_t n = total < cap ? total : cap;
+        if (e == cudaSuccess) {
+            total = h[0];
+            const int64_t n = std::min(total, cap);
+            if (n > 0) {
+                std::memcpy(indices, &h[1], sizeof(int64_t) * n);
+                std::memcpy(values, &h[1 + (size_t)cap], sizeof(double) * per * n);
+            }
+        }
+    } else {
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&total, counts + head, sizeof(int64_t), cudaMemcpyDeviceToHost, r->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
+        const int64_t n = std::min(total, cap);
         if (e == cudaSuccess && n > 0)
             e = cudaMemcpy(indices, idx_dev, sizeof(int64_t) * n, cudaMemcpyDeviceToHost);
         if (e == cudaSuccess && n > 0) e = cudaMemcpy(values, val_dev, sizeof(double) * per * n, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) rc = cuda_fail(e, "ket readout");
     }
-    if (counts) cudaFree(counts);
-    if (idx_dev) cudaFree(idx_dev);
-    if (val_dev) cudaFree(val_dev);
+    if (!keep) cudaFree(counts);
+    if (e != cudaSuccess) rc = cuda_fail(e, "ket readout");
     if (rc == QD_OK) *count = total;
     return rc;
 }
@@ -2043,7 +2061,7 @@ std::vector<std::pair<int, uint64_t>> batch_segments(const qd_batch *b, int c, u
 // appended to coef: ncoef hi entries, then ncoef lo entries.
 void split_coef(const GatePlan &g, BGate &bg, std::vector<float2> &coef) {
     const int n = bg.kind == 0 ? g.D * g.D : g.D;
-    const double *src = bg.kind == 0 ? g.U : g.lam;
+    const double *src = bg.kind == 0 ? g.U.data() : g.lam;
     bg.ncoef = (uint32_t)n;
     std::vector<float2> hi(n), lo(n);
     for (int k = 0; k < n; ++k) {
