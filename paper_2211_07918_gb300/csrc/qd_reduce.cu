@@ -47,16 +47,20 @@ __global__ void k_init(v2<T> *psi, uint64_t N, uint64_t idx) {
 // Two consecutive amplitudes at an even index i (16-byte aligned complex64
 // pairs), zeros beyond N.
 template <typename T, bool ALIGNED = true>
+__device__ __forceinline__ void load_pair(const v2<T> *__restrict__ psi, v2<T> *v) {
+    if constexpr (sizeof(T) == 4 && ALIGNED) {
+        const float4 q = *reinterpret_cast<const float4 *>(psi);
+        v[0] = make_float2(q.x, q.y);
+        v[1] = make_float2(q.z, q.w);
+    } else {
+        v[0] = psi[0];
+        v[1] = psi[1];
+    }
+}
+template <typename T, bool ALIGNED = true>
 __device__ __forceinline__ void load_pair(const v2<T> *__restrict__ psi, uint64_t i, uint64_t N, v2<T> *v) {
     if (i + 1 < N) {
-        if constexpr (sizeof(T) == 4 && ALIGNED) {
-            const float4 q = *reinterpret_cast<const float4 *>(psi + i);
-            v[0] = make_float2(q.x, q.y);
-            v[1] = make_float2(q.z, q.w);
-        } else {
-            v[0] = psi[i];
-            v[1] = psi[i + 1];
-        }
+        load_pair<T, ALIGNED>(psi + i, v);
     } else {
         v[0] = i < N ? psi[i] : mk<T>(T(0), T(0));
         v[1] = mk<T>(T(0), T(0));
@@ -74,7 +78,7 @@ template <typename T> constexpr int kSumGroup = sizeof(T) == 4 ? 8 : 4;
 // amplitudes.  With both squares of every amplitude in FP64 (conversions
 // included, five operations of the FP64 pipe each) the pipe's two lanes per
 // SM took 6x the time of the read on complex64 states.  3.4e8 amplitudes:
-// complex64 3154 -> 508 us (5.35 TB/s), complex128 1923 -> 899 us (6.05).
+// complex64 3154 -> 494 us (5.5 TB/s), complex128 1923 -> 868 us (6.26).
 template <typename T>
 __global__ void __launch_bounds__(kRedBlock, 5) k_norm_partial(const v2<T> *__restrict__ psi, uint64_t N,
                                                             double *__restrict__ part) {
@@ -84,8 +88,14 @@ __global__ void __launch_bounds__(kRedBlock, 5) k_norm_partial(const v2<T> *__re
     double acc = 0.0;
     for (uint64_t t = (uint64_t)blockIdx.x * tile; t < N; t += (uint64_t)gridDim.x * tile) {
         v2<T> v[G];
+        if (t + tile <= N) {
+            const v2<T> *p = psi + t + 2 * threadIdx.x;
 #pragma unroll
-        for (int k = 0; k < G / 2; ++k) load_pair<T>(psi, t + 2 * (k * kRedBlock + threadIdx.x), N, v + 2 * k);
+            for (int k = 0; k < G / 2; ++k) load_pair<T>(p + 2 * k * kRedBlock, v + 2 * k);
+        } else {
+#pragma unroll
+            for (int k = 0; k < G / 2; ++k) load_pair<T>(psi, t + 2 * (k * kRedBlock + threadIdx.x), N, v + 2 * k);
+        }
         acc += group_norm<T, G>(v);
     }
     acc = block_sum(acc, sh);
@@ -97,7 +107,7 @@ __global__ void __launch_bounds__(kRedBlock, 5) k_norm_partial(const v2<T> *__re
 // walk the state with step A, so that a thread meets one digit only and a
 // warp's loads are consecutive; every amplitude is read once.  One block sum
 // per digit at the end, hence only up to kPeriodDim levels.  3.4e8 complex64
-// amplitudes: 3248 -> 584 us (4.65 TB/s).
+// amplitudes: 3248 -> 524 us (5.2 TB/s; 584 with bounds checks in full tiles).
 constexpr uint32_t kPeriodMax = 16384;
 constexpr int kPeriodDim = 8;
 
@@ -111,10 +121,16 @@ __global__ void __launch_bounds__(kRedBlock, 5) k_digit_partial(const v2<T> *__r
     if (tid < A) {
         for (uint64_t i = tid; i < N; i += (uint64_t)G * A) {
             v2<T> v[G];
+            if (i + (uint64_t)(G - 1) * A < N) {
+                const v2<T> *p = psi + i;
 #pragma unroll
-            for (int k = 0; k < G; ++k) {
-                const uint64_t j = i + (uint64_t)k * A;
-                v[k] = j < N ? psi[j] : mk<T>(T(0), T(0));
+                for (int k = 0; k < G; ++k, p += A) v[k] = *p;
+            } else {
+#pragma unroll
+                for (int k = 0; k < G; ++k) {
+                    const uint64_t j = i + (uint64_t)k * A;
+                    v[k] = j < N ? psi[j] : mk<T>(T(0), T(0));
+                }
             }
             acc += group_norm<T, G>(v);
         }
@@ -132,7 +148,7 @@ __global__ void __launch_bounds__(kRedBlock, 5) k_digit_partial(const v2<T> *__r
 // most two runs): one division per tile instead of one per amplitude, whose
 // operations share the ALU pipe with the squares'.  3.4e8 complex64
 // amplitudes: 3245 us with FP64 squares, 784 with a division per amplitude,
-// 672 with LONG (4.05 TB/s).
+// 672 with LONG and 473 to 494 (5.6 TB/s) without bounds checks in full tiles.
 template <typename T, bool LONG>
 __global__ void __launch_bounds__(kRedBlock, 5) k_slice_partial(const v2<T> *__restrict__ psi, uint64_t M,
                                                                 FastDiv64 divs, uint64_t P,
@@ -147,6 +163,10 @@ __global__ void __launch_bounds__(kRedBlock, 5) k_slice_partial(const v2<T> *__r
         const uint64_t q = LONG ? fdiv(t, divs) : 0;
         const uint64_t left = LONG ? s - (t - q * s) : 0;  // of the tile's first run
         const v2<T> *first = psi + t + q * skip + off;
+        if (LONG && left >= tile && t + tile <= M) {  // one run
+#pragma unroll
+            for (int k = 0; k < G; ++k) v[k] = first[k * kRedBlock + threadIdx.x];
+        } else
 #pragma unroll
         for (int k = 0; k < G; ++k) {
             const uint32_t e = k * kRedBlock + threadIdx.x;
@@ -189,11 +209,21 @@ __global__ void __launch_bounds__(kRedBlock) k_overlap_partial(const v2<TA> *__r
     for (uint64_t t = (uint64_t)blockIdx.x * tile; t < N; t += (uint64_t)gridDim.x * tile) {
         v2<TA> x[G + F];
         v2<TB> y[G + F];
+        if (t + tile <= N) {
+            const v2<TA> *pa = a + t + 2 * threadIdx.x;
+            const v2<TB> *pb = b + t + 2 * threadIdx.x;
 #pragma unroll
-        for (int k = 0; k < (G + F) / 2; ++k) {
-            const uint64_t i = t + 2 * (k * kRedBlock + threadIdx.x);
-            load_pair<TA>(a, i, N, x + 2 * k);
-            load_pair<TB>(b, i, N, y + 2 * k);
+            for (int k = 0; k < (G + F) / 2; ++k) {
+                load_pair<TA>(pa + 2 * k * kRedBlock, x + 2 * k);
+                load_pair<TB>(pb + 2 * k * kRedBlock, y + 2 * k);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < (G + F) / 2; ++k) {
+                const uint64_t i = t + 2 * (k * kRedBlock + threadIdx.x);
+                load_pair<TA>(a, i, N, x + 2 * k);
+                load_pair<TB>(b, i, N, y + 2 * k);
+            }
         }
         double gr, gi;
         group_overlap<TA, TB, G>(x, y, gr, gi);
@@ -377,8 +407,8 @@ __device__ __forceinline__ uint64_t philox_word0(uint64_t c0, uint64_t key0) {
 // state and 8 bytes per amplitude written and read again.  A shot searches the
 // levels from the top and walks its 16 amplitudes.  Every level's prefix is
 // relative to its parent, and base + prefix > target decides at each.  One
-// shot from 3.4e8 complex64 amplitudes: 7582 us with the whole CDF, 636 us
-// (4.27 TB/s); a million shots: 8115 -> 908 us.
+// shot from 3.4e8 complex64 amplitudes: 7582 us with the whole CDF, 582 us
+// (4.67 TB/s); a million shots: 8115 -> 850 us.
 constexpr int kSampBlock = 256;
 constexpr int kSampPer = 16;                       // amplitudes per prefix entry
 constexpr int kSampChunk = kSampBlock * kSampPer;  // amplitudes per chunk
@@ -420,15 +450,24 @@ __global__ void __launch_bounds__(kSampBlock) k_samp_prefix(const v2<T> *__restr
     constexpr int R16 = kSampPer * (int)sizeof(v2<T>) / 16;  // 16-byte pieces of a row
     constexpr int A16 = 16 / (int)sizeof(v2<T>);             // amplitudes of a piece
     const uint64_t c0 = (uint64_t)blockIdx.x * kSampChunk;
+    if (c0 + kSampChunk <= N) {
 #pragma unroll
-    for (int k = 0; k < R16; ++k) {
-        const int e = k * kSampBlock + threadIdx.x;
-        const uint64_t i = c0 + (uint64_t)e * A16;
-        // pieces beyond N (and the odd half of the last one) are filled with zeros
-        const int bytes = i >= N ? 0 : (N - i >= A16 ? 16 : (int)sizeof(v2<T>));
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(rows + (e / R16) * kSampRow<T> + (e % R16) * 16);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(psi + (bytes ? i : 0)), "r"(bytes)
-                     : "memory");
+        for (int k = 0; k < R16; ++k) {
+            const int e = k * kSampBlock + threadIdx.x;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(rows + (e / R16) * kSampRow<T> + (e % R16) * 16);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(psi + c0 + e * A16) : "memory");
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R16; ++k) {
+            const int e = k * kSampBlock + threadIdx.x;
+            const uint64_t i = c0 + (uint64_t)e * A16;
+            // pieces beyond N (and the odd half of the last one) are filled with zeros
+            const int bytes = i >= N ? 0 : (N - i >= A16 ? 16 : (int)sizeof(v2<T>));
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(rows + (e / R16) * kSampRow<T> + (e % R16) * 16);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(psi + (bytes ? i : 0)), "r"(bytes)
+                         : "memory");
+        }
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
