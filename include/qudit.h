@@ -137,8 +137,11 @@ int qd_set_stream(qd_reg *reg, void *stream);
  * dimension D <= 32: 0 (default) lets the plan's cost model (analytic, or the
  * learned model for QD_PLAN_LEARNED) price both and take the cheaper, for D
  * >= 9; a value in 9..65 sends blocks of D >= value to the tensor cores
- * (exact BF16 slice products with FP32 accumulation) and smaller ones to the
- * CUDA-core dense kernels.  Blocks above 32 always run on the tensor cores. */
+ * (exact products of short digits with FP32 accumulation) and smaller ones,
+ * and single dense gates below it, to the CUDA-core dense kernels.  With the
+ * default, dense launches of 10 to 16 states run on the tensor cores.  Blocks
+ * above 32 always run there, and complex128 dense launches from 4 states on
+ * (2 and 3 on larger registers) whatever the value. */
 #define QD_TUNE_FUSE_KMAX 2
 #define QD_TUNE_FUSE_DMAX 3
 #define QD_TUNE_TC_MIN_D 4
@@ -440,7 +443,7 @@ int qd_set_cost_model(qd_reg *reg, qd_model *model);
 /* Kernel forms of one launch (launch feature 10). */
 #define QD_FORM_MONO 0       /* one permutation / diagonal gate */
 #define QD_FORM_DENSE 1      /* one dense gate */
-#define QD_FORM_BLOCK 2      /* fused block, CUDA-core dense kernel (D <= 32) */
+#define QD_FORM_BLOCK 2      /* fused block, dense-gate kernels (D <= 32; complex64 of 10 to 16 states, see QD_TUNE_TC_MIN_D, and complex128 on the tensor cores) */
 #define QD_FORM_BLOCK_TC 3   /* fused block, tensor-core kernel (complex64, 9 <= D <= 64) */
 #define QD_FORM_DIAG_RUN 4   /* run of diagonal gates through one table */
 #define QD_FORM_DENSE_RUN 5  /* dense part (<= 16 states) followed by a diagonal run */

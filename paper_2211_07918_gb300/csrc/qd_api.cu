@@ -305,6 +305,7 @@ int plan_gate(const qd_reg *r, const double *M, const Acting &a, bool diag_only,
     g.D = D;
     g.N = (uint64_t)r->N;
     g.wide = r->index64 != 0;
+    g.cuda_cores = D < r->tc_min_d;
     g.pow2 = all_pow2(r);
     // matrix / classification
     if (force_dense) {  // the dense kernels, whatever the matrix (a dense part with a table epilogue)

@@ -31,6 +31,7 @@ struct GatePlan {
     int32_t D = 0;
     uint64_t N = 0;  // register size (selects 32- or 64-bit index arithmetic)
     bool wide = false;  // 64-bit index arithmetic below 2^31 too (QD_TUNE_INDEX64)
+    bool cuda_cores = false;  // complex64: below QD_TUNE_TC_MIN_D, kept off the tensor cores
     bool pow2 = false;  // every qudit dimension of the register is a power of two
 
     // --- direct mode: one thread per group --------------------------------

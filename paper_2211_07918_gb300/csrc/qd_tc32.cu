@@ -440,7 +440,7 @@ bool tc_matrix_ordinary(const GatePlan &g, int low, int high) {
 bool tc32_takes(const GatePlan &g, bool block) {
     if (g.kind != Kind::Dense || g.mode != Mode::Direct || g.tab || g.D < kTcMinD || g.D > kMaxDim) return false;
     if (!block) {
-        if (g.D == kTcMinD) return false;
+        if (g.D == kTcMinD || g.cuda_cores) return false;
         bool consecutive = g.D == kMaxDim;
         for (int j = 0; j < g.D && consecutive; ++j) consecutive = g.off[j] >= 0 && g.off[j] < g.D;
         if (consecutive) return false;
