@@ -193,10 +193,22 @@ __host__ __device__ constexpr int direct_min_blocks() {
     return !kSplit<T> ? 1 : MD >= 32 ? (DENSE ? 2 : 3) : (DENSE && MD == 8 ? 3 : 4);
 }
 
+// The chained kernels (qd_launch.cuh).  5 and 6 states are left out: the two
+// instructions alone made them slower on mid-sized states (D = 5, 2 Mi
+// complex64 amplitudes: 4.02 -> 4.33 us unchained).
+template <int MD>
+constexpr bool kDenseChains = MD <= 4 || MD == 8;
+template <typename T>
+uint64_t chain_limit(int D) {
+    return kSplit<T> && D == 3 ? kChainL2Bytes : kChainBytes;
+}
+
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256, (direct_min_blocks<T, MD, true>())) k_dense_direct(const __grid_constant__ DenseDirectArgs<T, I, MD> a) {
-    chain_release();
-    chain_wait();
+    if constexpr (kDenseChains<MD>) {
+        chain_release();
+        chain_wait();
+    }
     constexpr int UN = direct_unroll<T, I, MD>();
     const int D = EX ? MD : a.D;
     const I step = (I)gridDim.x * blockDim.x;
@@ -378,8 +390,10 @@ __host__ __device__ constexpr int table_min_blocks() {
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256, (table_min_blocks<T, I, MD>()))
     k_dense_table(const __grid_constant__ DenseTableArgs<T, I, MD> a) {
-    chain_release();
-    chain_wait();
+    if constexpr (MD <= 4) {
+        chain_release();
+        chain_wait();
+    }
     constexpr int UN = MD <= 4 ? 2 : 1;
     constexpr int TB = MD <= 4 ? MD : 2;  // outputs whose entries are loaded together
     using Entry = typename TabEntry<T>::type;
@@ -517,8 +531,10 @@ __device__ __forceinline__ void tile_store(const TileGeo<I> &t, v2<T> *psi, uint
 
 template <typename T, typename I, int MD, bool EX>
 __global__ void __launch_bounds__(256) k_dense_tile(const __grid_constant__ DenseTileArgs<T, I, MD> a) {
-    chain_release();
-    chain_wait();
+    if constexpr (MD <= 4) {
+        chain_release();
+        chain_wait();
+    }
     extern __shared__ __align__(16) unsigned char smraw[];
     const TileGeo<I> &t = a.t;
     const int D = EX ? MD : a.D;
@@ -719,7 +735,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
         auto fn = k_dense_direct<T, I, MD, EX>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
+        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), kDenseChains<MD> ? chain_limit<T>(g.D) : 0, a);
     }
     DenseTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -736,7 +752,7 @@ cudaError_t launch_dense(const GatePlan &g, void *psi, int sm_count, cudaStream_
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), a);
+    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), MD <= 4 ? chain_limit<T>(g.D) : 0, a);
 }
 
 // A permutation with phases whose moved members are few (a fused Toffoli
@@ -775,7 +791,7 @@ cudaError_t launch_mono_compact(const GatePlan &g, void *psi, int sm_count, cuda
     auto fn = k_mono_direct<T, I, MD>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
+    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), chain_limit<T>(g.D), a);
 }
 
 template <typename T, typename I, int MD>
@@ -797,7 +813,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
         auto fn = k_mono_direct<T, I, MD>;
         const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
         if (grid <= 0) return cudaSuccess;
-        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
+        return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), chain_limit<T>(g.D), a);
     }
     MonoTileArgs<T, I, MD> a;
     a.psi = static_cast<v2<T> *>(psi);
@@ -817,7 +833,7 @@ cudaError_t launch_mono(const GatePlan &g, void *psi, int sm_count, cudaStream_t
     if (e != cudaSuccess) return e;
     const int grid = grid_of(g.R_tiles, g.tpc, sm_count, occupancy_blocks((const void *)fn, kBlock, smem));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), a);
+    return launch_chained(fn, grid, kBlock, smem, s, g.N * sizeof(v2<T>), chain_limit<T>(g.D), a);
 }
 
 template <typename T, typename I, int MD, bool EX>
@@ -851,7 +867,7 @@ cudaError_t launch_dense_table(const GatePlan &g, void *psi, int sm_count, cudaS
     auto fn = k_dense_table<T, I, MD, EX>;
     const int grid = grid_of(g.R, kBlock, sm_count, occupancy_blocks((const void *)fn, kBlock, 0));
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), a);
+    return launch_chained(fn, grid, kBlock, 0, s, g.N * sizeof(v2<T>), MD <= 4 ? chain_limit<T>(g.D) : 0, a);
 }
 
 template <typename T, typename I>

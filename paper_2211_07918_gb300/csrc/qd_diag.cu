@@ -158,18 +158,18 @@ cudaError_t diag_table_apply(void *psi, int prec, uint64_t N, uint64_t s_qa, uin
     if (N < (uint64_t(1) << 31) && !wide) {
         const FastDiv32 a = make_fastdiv32((uint32_t)s_qa), t = make_fastdiv32((uint32_t)TS);
         if (prec == 1)
-            e = launch_chained(k_diag_apply_f32<uint32_t>, grid, kDiagBlock, 0, s, 8 * N, static_cast<float2 *>(psi), (uint32_t)N, a, t,
+            e = launch_chained(k_diag_apply_f32<uint32_t>, grid, kDiagBlock, 0, s, 8 * N, kChainBytes, static_cast<float2 *>(psi), (uint32_t)N, a, t,
                                                                    static_cast<const float4 *>(tab));
         else
-            e = launch_chained(k_diag_apply_f64<uint32_t>, grid, kDiagBlock, 0, s, 16 * N, static_cast<double2 *>(psi), (uint32_t)N, a, t,
+            e = launch_chained(k_diag_apply_f64<uint32_t>, grid, kDiagBlock, 0, s, 16 * N, kChainBytes, static_cast<double2 *>(psi), (uint32_t)N, a, t,
                                                                    static_cast<const double2 *>(tab));
     } else {
         const FastDiv64 a = make_fastdiv64(s_qa), t = make_fastdiv64(TS);
         if (prec == 1)
-            e = launch_chained(k_diag_apply_f32<uint64_t>, grid, kDiagBlock, 0, s, 8 * N, static_cast<float2 *>(psi), N, a, t,
+            e = launch_chained(k_diag_apply_f32<uint64_t>, grid, kDiagBlock, 0, s, 8 * N, kChainBytes, static_cast<float2 *>(psi), N, a, t,
                                                                    static_cast<const float4 *>(tab));
         else
-            e = launch_chained(k_diag_apply_f64<uint64_t>, grid, kDiagBlock, 0, s, 16 * N, static_cast<double2 *>(psi), N, a, t,
+            e = launch_chained(k_diag_apply_f64<uint64_t>, grid, kDiagBlock, 0, s, 16 * N, kChainBytes, static_cast<double2 *>(psi), N, a, t,
                                                                    static_cast<const double2 *>(tab));
     }
     return e;

@@ -9,10 +9,24 @@
 // come onto the SMs: at its start, or, if it allocates TMEM, after that (the
 // next kernel's blocks must not take TMEM that this kernel's still need).
 // Kernels and copies launched without the attribute wait for completion as
-// usual.  Only states that fit the L2 cache are chained: on large
-// ones the latency is nothing against the pass (direct gate calls on 4.3e8
-// amplitudes 10.80 ms chained, 10.62 not).  Measured: 500 gates on 4.8e6 complex64 amplitudes in L2 3747 -> 3567
-// us; 40 gates on 324 complex128 amplitudes, planned, run and read, 497 -> 398 us.
+// usual.
+//
+// Chaining pays where a launch is mostly latency, and costs where the early
+// blocks take issue slots from the pass still running.  Per gate, 40 gates of
+// one kind on complex64 states, unchained -> chained, us:
+//   amplitudes      1 Ki          16 Ki         128 Ki        1 Mi        4 Mi
+//   X,  D = 2   1.56 -> 1.35  1.58 -> 1.50  1.76 -> 1.90  3.05 -> 2.94  7.14 -> 7.41
+//   dense D = 3 1.71 -> 1.35  1.71 -> 1.47  1.76 -> 1.60  2.85 -> 2.63  6.61 -> 6.38
+//   dense D = 4 1.86 -> 1.51  1.91 -> 1.61  1.96 -> 1.99  3.92 -> 3.87 10.23 -> 9.98 (256 Ki: 2.12 -> 2.82)
+//   dense D = 8 2.17 -> 1.71  2.64 -> 2.18  2.68 -> 2.67  5.09 -> 4.42
+//   D = 10, tensor cores      3.92 -> 3.65  3.96 -> 3.66  6.73 -> 6.49 13.26 -> 12.92
+// So every kernel chains on states of kChainBytes, complex64 gates of three
+// states (complex128, 128 Ki: 2.6 -> 3.7) and the tensor-core kernels on all
+// states that fit L2 (kChainL2Bytes; on larger
+// ones it is a loss: direct gate calls on 4.3e8 amplitudes 10.80 ms chained,
+// 10.62 not), and the CUDA-core dense kernels above 8 states never (D = 9:
+// 3.65 -> 3.73 at 16 Ki, 3.61 -> 4.43 at 256 Ki, 4.64 -> 7.01 at 1 Mi).
+// 40 gates on 324 complex128 amplitudes, planned, run and read: 497 -> 398 us.
 #pragma once
 #include <cstdint>
 #include <utility>
@@ -24,11 +38,13 @@ namespace qd {
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-constexpr uint64_t kChainBytes = uint64_t(128) << 20;
+constexpr uint64_t kChainBytes = uint64_t(256) << 10;
+constexpr uint64_t kChainL2Bytes = uint64_t(128) << 20;
 
-// state_bytes: the size of the state the kernel works on.
+// state_bytes: the size of the state the kernel works on; limit: up to which
+// it is chained (0: never).
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t s, uint64_t state_bytes,
+inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t s, uint64_t state_bytes, uint64_t limit,
                                   A &&...args) {
     cudaLaunchConfig_t c{};
     c.gridDim = dim3((unsigned)grid);
@@ -39,7 +55,7 @@ inline cudaError_t launch_chained(void (*fn)(P...), int grid, int block, size_t 
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
-    c.numAttrs = s && state_bytes <= kChainBytes ? 1 : 0;  // (the legacy default stream orders whole kernels)
+    c.numAttrs = s && state_bytes <= limit ? 1 : 0;  // (the legacy default stream orders whole kernels)
     return cudaLaunchKernelEx(&c, fn, std::forward<A>(args)...);
 }
 

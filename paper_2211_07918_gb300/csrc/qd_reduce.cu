@@ -597,8 +597,8 @@ int grid_for(uint64_t n, int block, int sm_count, int per_sm) {
 
 cudaError_t init_basis(void *psi, int prec, uint64_t N, uint64_t idx, int sm_count, cudaStream_t s) {
     const int g = grid_for(N, 256, sm_count, 8);
-    if (prec == 1) return launch_chained(k_init<float>, g, 256, 0, s, 8 * N, static_cast<float2 *>(psi), N, idx);
-    return launch_chained(k_init<double>, g, 256, 0, s, 16 * N, static_cast<double2 *>(psi), N, idx);
+    if (prec == 1) return launch_chained(k_init<float>, g, 256, 0, s, 8 * N, kChainBytes, static_cast<float2 *>(psi), N, idx);
+    return launch_chained(k_init<double>, g, 256, 0, s, 16 * N, kChainBytes, static_cast<double2 *>(psi), N, idx);
 }
 
 // the resident blocks of the sums (256 threads of at most 48 registers)

@@ -626,7 +626,7 @@ static cudaError_t launch_tc_im(const GatePlan &g, void *psi, int sm_count, int3
     const uint64_t cap = (uint64_t)sm_count * occ;
     const int grid = (int)(tiles < cap ? tiles : cap);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, C::THREADS, (size_t)smem, s, 8 * g.N, a);
+    return launch_chained(fn, grid, C::THREADS, (size_t)smem, s, 8 * g.N, kChainL2Bytes, a);
 }
 
 template <typename I>

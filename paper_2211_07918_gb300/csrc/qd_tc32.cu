@@ -377,7 +377,7 @@ cudaError_t launch_fn(const Tc32Args<I> &a, uint64_t N, int sm_count, cudaStream
     const uint64_t tiles = ((uint64_t)a.R + kRows - 1) / kRows;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * kPerSm);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, kThreads, kData, s, 8 * N, a);
+    return launch_chained(fn, grid, kThreads, kData, s, 8 * N, kChainL2Bytes, a);
 }
 
 // Exponent field of the matrix' largest part.

@@ -551,7 +551,7 @@ cudaError_t launch_tab(const GatePlan &g, void *psi, int sm_count, int32_t *err,
     const uint64_t tiles = (g.R + C::PER_TILE - 1) / C::PER_TILE;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * C::PER_SM);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, a, tb);
+    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, kChainL2Bytes, a, tb);
 }
 
 template <typename I, int NP, int GD>
