@@ -154,7 +154,7 @@ cudaError_t launch_plan(const qd_reg *r, const GatePlan &g) {
         return diag_table_apply(r->psi, r->prec, (uint64_t)r->N, g.tab_div, g.tab_size, g.tab, r->sm_count, r->stream,
                                 g.wide);
     if (r->prec == QD_C64) {
-        if (tc32_takes(g, false)) return launch_dense_tc32(g, r->psi, r->sm_count, r->dev_err, r->stream);
+        if (tc32_takes(g, false, r->sm_count)) return launch_dense_tc32(g, r->psi, r->sm_count, r->dev_err, r->stream);
         return launch_gate_f32(g, r->psi, r->sm_count, r->stream);
     }
     if (tc64_takes(g)) return launch_dense_tc64(g, r->psi, r->sm_count, r->dev_err, r->stream);
@@ -1018,7 +1018,7 @@ int plan_block_tc(const qd_reg *r, const FuseBlock &b, GatePlan &g, std::vector<
     if (b.D <= 16) {  // qd_tc32.cu, its matrix in the launch's arguments; no terms
         g.U = b.M;
         g.mode = Mode::Direct;
-        const bool takes = tc32_takes(g, true);
+        const bool takes = tc32_takes(g, true, r->sm_count);
         g.mode = Mode::Tensor;
         if (takes) return QD_OK;
     }

@@ -35,7 +35,7 @@ cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_
 // (qd_tc32.cu): whether the kernel takes a launch (direct geometry, matrix
 // entries of ordinary size; for a single gate or a block priced on the CUDA
 // cores, the shapes at which it is the faster one), and the launch.
-bool tc32_takes(const GatePlan &g, bool block);
+bool tc32_takes(const GatePlan &g, bool block, int sm_count);
 cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
 
 // Whether the exponent field of every matrix row's largest entry lies in

@@ -437,10 +437,20 @@ bool tc_matrix_ordinary(const GatePlan &g, int low, int high) {
     return true;
 }
 
-bool tc32_takes(const GatePlan &g, bool block) {
+// A single gate leaves the tensor cores where its groups fill one wave of the
+// CUDA-core kernel (512 threads an SM, one group each) and more than two tiles
+// an SM here.  us per gate, CUDA cores / here, states in L2:
+//   groups    32 Ki        64 Ki        76 Ki        80 Ki       112 Ki       160 Ki
+//   D = 10  4.73 / 4.59  5.04 / 6.38  5.04 / 6.63  6.78 / 6.94  7.09 / 7.50 10.42 / 9.42
+//   D = 12  5.50 / 4.73  5.86 / 6.69  5.89 / 6.88  7.84 / 7.19  7.96 / 7.70 11.95 / 9.90
+//   D = 16  6.62 / 5.09  7.14 / 7.35  7.14 / 7.49 10.06 / 7.93 10.26 / 8.53 15.43 / 11.04
+// (at D = 10 the second wave, of 256 threads an SM, is the better one too).
+bool tc32_takes(const GatePlan &g, bool block, int sm_count) {
     if (g.kind != Kind::Dense || g.mode != Mode::Direct || g.tab || g.D < kTcMinD || g.D > kMaxDim) return false;
     if (!block) {
         if (g.D == kTcMinD || g.cuda_cores) return false;
+        const uint64_t sms = (uint64_t)sm_count;
+        if (g.R > 256 * sms && g.R <= (g.D == 10 ? 768 : 512) * sms) return false;
         bool consecutive = g.D == kMaxDim;
         for (int j = 0; j < g.D && consecutive; ++j) consecutive = g.off[j] >= 0 && g.off[j] < g.D;
         if (consecutive) return false;
