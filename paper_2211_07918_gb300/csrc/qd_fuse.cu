@@ -246,7 +246,12 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
             if (!c128 && D > 9.5 && D < 16.5) t_cmp = std::min(t_cmp, touched * 5.1e-11 / D);
         }
     }
-    return std::max(t_mem, t_cmp) + 4.0e-6;
+    // a launch, and what the complex64 dense kernels take longer than a mono
+    // kernel on a state of a few amplitudes (1.5 us: 0.1 at D = 4, 0.6 at D = 8,
+    // 2.0 to 2.5 from D = 9 on): without it a plan of a small register takes a
+    // dense launch where a mono one is as good
+    const double setup = !dense || c128 ? 0.0 : D < 8.5 ? 0.07e-6 * D : 2.0e-6;
+    return std::max(t_mem, t_cmp) + setup + 4.0e-6;
 }
 
 double segment_cost(const std::vector<FuseGate> &gates, int first, int last, const RegisterShape &reg,
