@@ -214,8 +214,10 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     // feature 11: log2 of the control-slice fraction, or (dense + table) of the table entries
     const double touched = dense_table ? (double)reg.N : (double)reg.N * std::exp2((double)lf.f[11]);
     const double b = c128 ? 16.0 : 8.0;
-    // 5.4 TB/s: what the memory-bound dense kernels move on large registers
-    double t_mem = 2.0 * touched * b / (dense ? 5.4e12 : 5.0e12);
+    // 5.4 TB/s: what the memory-bound dense and mono kernels move on large
+    // registers (with 5.0 for mono a 2^32 Fourier ladder took a dense D = 16
+    // launch of 13.0 ms for a mono one of 5.9: 239.7 -> 244.8 ms)
+    double t_mem = 2.0 * touched * b / (table ? 5.0e12 : 5.4e12);
     if (table) t_mem += std::exp2((double)lf.f[0]) * 16.0 / 5.0e12;
     if (dense_table) t_mem += std::exp2((double)lf.f[11]) * 16.0 / 5.0e12;
     // complex128 dense kernels: the CUDA cores take 4 D DFMA per amplitude; the
@@ -234,16 +236,16 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     if (dense && !table && !dense_table) {
         if (!c128 && block) {
             // fused block on the tensor cores: measured on GB300 it moves about
-            // 5.3 TB/s at D = Dp (4.95 above 32), less in proportion to the
-            // padding; up to D = 16 (qd_tc32.cu) 5.0 TB/s at full rows of 16 slots
+            // 5.3 TB/s at D = Dp (5.1 up to 24, 4.95 above 32), less in proportion
+            // to the padding; up to D = 16 (qd_tc32.cu) 5.4 TB/s at full rows of 16 slots
             const double Dp = D <= 32 ? std::ceil(D / 8.0) * 8.0 : std::ceil(D / 16.0) * 16.0;
-            t_cmp = D < 16.5 ? touched * 5.1e-11 / D : 2.0 * touched * b / ((D <= 32 ? 5.3e12 : 4.95e12) * D / Dp);
+            t_cmp = D < 16.5 ? touched * 4.7e-11 / D : 2.0 * touched * b / ((D <= 24.5 ? 5.1e12 : D <= 32.5 ? 5.3e12 : 4.95e12) * D / Dp);
         } else {
             // complex64 with hi+lo coefficients: hidden under the memory pass up to
             // D = 8, then 8 D FFMA per amplitude plus index work (packed at D = 9);
             // from D = 10 to 16 the tensor cores (qd_tc32.cu) at rows of 16 slots
             t_cmp = c128 ? t_c128 : D < 8.5 ? 0.0 : touched * (8.0 * D + 24.0) / (D < 9.5 ? 2.4e13 : 2.0e13);
-            if (!c128 && D > 9.5 && D < 16.5) t_cmp = std::min(t_cmp, touched * 5.1e-11 / D);
+            if (!c128 && D > 9.5 && D < 16.5) t_cmp = std::min(t_cmp, touched * 4.7e-11 / D);
         }
     }
     // a launch, and what the complex64 dense kernels take longer than a mono
