@@ -141,7 +141,8 @@ int qd_set_stream(qd_reg *reg, void *stream);
  * and single dense gates below it, to the CUDA-core dense kernels.  With the
  * default, dense launches of 10 to 16 states run on the tensor cores.  Blocks
  * above 32 always run there, and complex128 dense launches from 4 states on
- * (2 and 3 on larger registers) whatever the value. */
+ * (2 and 3 on larger registers; for the matrices see qd_apply) whatever the
+ * value. */
 #define QD_TUNE_FUSE_KMAX 2
 #define QD_TUNE_FUSE_DMAX 3
 #define QD_TUNE_TC_MIN_D 4
@@ -159,7 +160,14 @@ int qd_set_tuning(qd_reg *reg, int32_t key, int64_t value);
  * ctrl_levels (NULL or -1 entries: d_c - 1).  The matrix is classified on
  * the host: a diagonal or a permutation-with-phases matrix runs the
  * data-movement kernels, anything else the dense kernels.  No check of
- * unitarity.  Errors: QD_ERR_ARG, QD_ERR_DIM (D > QD_MAX_D), QD_ERR_OVERLAP. */
+ * unitarity.  Errors: QD_ERR_ARG, QD_ERR_DIM (D > QD_MAX_D), QD_ERR_OVERLAP.
+ * Accuracy of a complex128 dense matrix U on a group v of D amplitudes: the
+ * tensor cores take matrices that fall into full parts (any two rows couple
+ * the same members or none in common, a row's non-zero entries lie within
+ * 2^10 of each other); output i is then off by at most
+ * 4 D 2^-53 max_j |u_ij| max_j |v_j|, the maxima over the members j that row i
+ * couples.  Other matrices are sums of rounded products, off by at most
+ * 4 D 2^-53 sum_j |u_ij| |v_j|. */
 int qd_apply(qd_reg *reg, const double *matrix, const int32_t *targets, int32_t k,
              const int32_t *controls, const int32_t *ctrl_levels, int32_t nc);
 

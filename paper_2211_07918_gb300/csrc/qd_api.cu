@@ -913,6 +913,7 @@ int collect_gates(const qd_reg *r, const qd_gate *gates, int32_t ngates, std::ve
                 bool ident = g.kind == Kind::Mono;  // a permutation with phases whose permutation is the identity
                 for (int j = 0; ident && j < a.D; ++j) ident = g.src[j] == j;
                 fg.back().diag = ident;
+                fg.back().fp64 = r->prec == QD_C128 && g.kind == Kind::Dense && !tc64_matrix(g.U.data(), g.D);
                 orig.push_back(gt);
             }
         }

@@ -6,6 +6,7 @@
 #include <map>
 
 #include "qd_fuse.h"
+#include "qd_tc.h"
 
 namespace qd {
 
@@ -229,7 +230,7 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     if (c128) {
         const double Dp = std::ceil(D / 8.0) * 8.0;
         const double t_tc = touched * (D <= 4.5 ? 8.2e-12 : D <= 16.5 ? 9.6e-12 * (1.0 + 0.65 * (Dp - D) / Dp) : 15.0e-12) + 1.0e-6;
-        t_c128 = std::min(t_c128, t_tc);
+        if (!lf.fp64) t_c128 = std::min(t_c128, t_tc);
     }
     double t_cmp = table ? touched * 40.0 / 2.0e13 : 0.0;  // index arithmetic per amplitude
     if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : D <= 4.5 ? 0.0 : touched * (8.0 * D + 64.0) / 2.0e13;
@@ -267,8 +268,16 @@ double segment_cost(const std::vector<FuseGate> &gates, int first, int last, con
             Dt /= reg.dims[g.acting[m]];
         }
         if (kind_out) *kind_out = g.mono ? kKernelMono : kKernelDense;
-        return cost(launch_features(reg, g.acting, Dt, g.mono ? kKernelMono : kKernelDense, frac));
+        LaunchFeatures lf = launch_features(reg, g.acting, Dt, g.mono ? kKernelMono : kKernelDense, frac);
+        lf.fp64 = g.fp64;
+        return cost(lf);
     }
+    // which complex128 kernel takes the product of gates a..b (10 us of host time per gate)
+    auto on_fp64 = [&](int a, int b) {
+        if (reg.precision == 1) return false;
+        const FuseBlock blk = build_block(gates, a, b, reg.dims);
+        return blk.D > kMaxD || !tc64_matrix(blk.M.data(), blk.D);
+    };
     const std::vector<int> s = union_qudits(gates, first, last);
     const int64_t D = dim_of(s, reg.dims);
     // a product of permutations with phases is one: it runs on the mono
@@ -288,9 +297,9 @@ double segment_cost(const std::vector<FuseGate> &gates, int first, int last, con
     double best = std::numeric_limits<double>::infinity();
     for (int k = 0; k < nk; ++k) {
         const int kind = kinds[k];
-        const double c = kind == kKernelDiagTable
-                             ? cost(launch_features(reg, s, (int)diag_table_size(reg, s), kind, 1.0))
-                             : cost(launch_features(reg, s, (int)D, kind, 1.0));
+        LaunchFeatures lf = launch_features(reg, s, kind == kKernelDiagTable ? (int)diag_table_size(reg, s) : (int)D, kind, 1.0);
+        lf.fp64 = kind == kKernelBlock && on_fp64(first, last);
+        const double c = cost(lf);
         if (c < best) {
             best = c;
             if (kind_out) *kind_out = kind;
@@ -298,8 +307,9 @@ double segment_cost(const std::vector<FuseGate> &gates, int first, int last, con
     }
     const DenseTableSplit dt = dense_table_split(gates, first, last, reg, kmax);
     if (dt.ok) {
-        const double c =
-            cost(launch_features(reg, dt.dense_q, (int)dt.dense_D, kKernelDenseTable, (double)dt.table));
+        LaunchFeatures lf = launch_features(reg, dt.dense_q, (int)dt.dense_D, kKernelDenseTable, (double)dt.table);
+        lf.fp64 = on_fp64(first, dt.split);
+        const double c = cost(lf);
         if (c < best) {
             best = c;
             if (kind_out) *kind_out = kKernelDenseTable;

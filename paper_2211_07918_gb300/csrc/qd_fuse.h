@@ -23,6 +23,7 @@ struct FuseGate {
     int Dact = 1;
     bool mono = false;      // the original gate is a permutation with phases
     bool diag = false;      // ... and its permutation is the identity (a diagonal gate)
+    bool fp64 = false;      // a dense gate whose matrix the complex128 tensor-core kernel does not take
     int nc = 0;             // number of controls in `acting`
 };
 
@@ -37,6 +38,7 @@ struct FuseBlock {
 constexpr int kFeatures = 12;
 struct LaunchFeatures {
     float f[kFeatures];
+    bool fp64 = false;  // complex128: the launch's matrix keeps it on the FP64 pipe (tc64_matrix)
 };
 
 struct RegisterShape {

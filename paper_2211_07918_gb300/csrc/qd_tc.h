@@ -40,6 +40,22 @@ cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_
 
 // Whether the exponent field of every matrix row's largest entry lies in
 // [low, high] (rows of zeros aside).
-bool tc_matrix_ordinary(const GatePlan &g, int low, int high);
+bool tc_matrix_ordinary(const double *U, int D, int low, int high);
+
+// What a dense matrix mixes: row i takes the members of_row[i]; member j
+// belongs to the part of_col[j]; one: a single part of all members.
+struct TcCouples {
+    bool one;
+    uint32_t of_row[kMaxD], of_col[kMaxD];
+};
+// False where the parts are not told apart by the zeros of the rows (two rows
+// share some of their members, not all) or the exponents of a row's entries
+// differ by more than `spread`: an output may then be much smaller than the
+// largest member of its part for other reasons than cancellation, and a scale
+// per part does not hold it to the accuracy of a sum of rounded products.
+bool tc_couples(const double *U, int D, int spread, TcCouples &c);
+
+// Whether k_dense_tc64 takes a launch with this matrix.
+bool tc64_matrix(const double *U, int D);
 
 }  // namespace qd

@@ -424,12 +424,12 @@ cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, c
 
 }  // namespace
 
-bool tc_matrix_ordinary(const GatePlan &g, int low, int high) {
-    for (int i = 0; i < g.D; ++i) {
+bool tc_matrix_ordinary(const double *U, int D, int low, int high) {
+    for (int i = 0; i < D; ++i) {
         int top = 0;
-        for (int k = 0; k < 2 * g.D; ++k) {
+        for (int k = 0; k < 2 * D; ++k) {
             uint64_t b;
-            std::memcpy(&b, &g.U[2 * i * g.D + k], 8);
+            std::memcpy(&b, &U[2 * i * D + k], 8);
             top = std::max(top, (int)((b >> 52) & 0x7ff));
         }
         if (top && (top < low || top > high)) return false;
@@ -456,7 +456,7 @@ bool tc32_takes(const GatePlan &g, bool block, int sm_count) {
         if (consecutive) return false;
     }
     const int top = matrix_top(g);
-    return top >= kMatExLow && top <= kMatExHigh && tc_matrix_ordinary(g, top - kMatRows, top);
+    return top >= kMatExLow && top <= kMatExHigh && tc_matrix_ordinary(g.U.data(), g.D, top - kMatRows, top);
 }
 
 cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {

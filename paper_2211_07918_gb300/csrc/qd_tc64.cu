@@ -18,6 +18,17 @@
 // 0.6 (D = 2) to 0.3 (D = 32) of that of the FP64 multiply-adds, which round
 // 4 D times.
 //
+// These errors are relative to the largest member on the scale, while a sum of
+// rounded products is off relative to its own terms: an output that takes only
+// small members, or a large one by a small entry, would lose the digits below
+// 2^-55 of the scale.  So members that the matrix does not couple never share
+// one: a matrix that falls into parts (a controlled gate or a gate on one of
+// its qudits, as a block; tc_couples) has a scale for each part of each group
+// (PARTS), and matrices whose rows share some of their members, or hold
+// entries more than 2^10 apart, stay on the FP64 pipe.  With a single scale,
+// the half of diag(R, R) at 1e-12 of the other was off by 1e-6 of itself; with
+// two by 4e-16.
+//
 // A tile is 128 rows of 8 NP amplitude slots (K = 16 NP): one group of D
 // amplitudes per row, spread evenly over its 2 NP threads, or for D <= 4
 // several groups side by side with a block-diagonal matrix.  The matrix digits
@@ -40,7 +51,13 @@
 // 1561 -> 337, D = 9 2349 -> 413, D = 27 about 6900 -> 520; D = 9 with a
 // diagonal run 4403 -> 554; 4,608 amplitudes at D = 9: 25.2 -> 5.8 us, at
 // D = 32: 304 -> 14 us (one thread's serial chain of FP64 operations before).
+// Matrices of parts (a gate on the lower qudit; controlled), single scale ->
+// a scale per part (the loop over a part's members, uniform in a warp, and up
+// to two scales per amplitude): D = 4 278 -> 471; 457 (a group per row instead
+// of four; CUDA cores 1039), D = 9 413 -> 495; 463 (2321), D = 16 356 -> 449;
+// 416 (4113), D = 27 473 -> 618; 545 (8365).
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -66,6 +83,8 @@ constexpr int kSlots = 4;      // amplitude slots of a thread (one 16-byte piece
 constexpr int kRowExLow = 400, kRowExHigh = 1900;
 // ... and of a matrix row's largest entry (checked on the host).
 constexpr int kMatExLow = 923, kMatExHigh = 1123;
+// ... and how far below it the row's smallest non-zero entry may lie.
+constexpr int kMatSpread = 10;
 
 template <typename I>
 struct Tc64Args {
@@ -94,6 +113,12 @@ template <typename I> struct Tc64Tab<I, true> {
     uint32_t carry, tsmask;
     const double2 *tab;
 };
+
+// Masks of the members that the matrix mixes, for matrices that fall into
+// parts (TcCouples): of input member j with the others of its part, and of the
+// members that go into output i.  Every part has a scale of its own.
+template <bool PARTS> struct Tc64Parts {};
+template <> struct Tc64Parts<true> { uint32_t in[kMaxD], out[kMaxD]; };
 
 // Scale exponent (FP64 bias, of 2^(E - 1022)) of a group or matrix row whose
 // largest part has the leading word top: parts are below 1 - 2^-7 of the
@@ -283,21 +308,25 @@ __device__ __forceinline__ void issue_digit(uint32_t tmem, uint64_t dx, uint64_t
 // launch's time (D = 3: 310 -> 286 us on 3.4e7 amplitudes; with a group per
 // row, whose CTAs wait at one more barrier, the shares were better: D = 9 415
 // against 485 us).
-template <typename I, int NP, int GD, bool TAB>
+template <typename I, int NP, int GD, bool TAB, bool PARTS>
 __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER_SM)
-    k_dense_tc64(const __grid_constant__ Tc64Args<I> a, const __grid_constant__ Tc64Tab<I, TAB> tb) {
+    k_dense_tc64(const __grid_constant__ Tc64Args<I> a, const __grid_constant__ Tc64Tab<I, TAB> tb,
+                 const __grid_constant__ Tc64Parts<PARTS> pt) {
     using C = Tc64Cfg<NP, GD>;
     using S = Slot<I, NP, GD>;
     constexpr int TG = C::TG;
     constexpr int GS = GD ? GD : kSlots;  // slots of a group in this thread
     constexpr bool QUEUE = GD != 0;
+    static_assert(!PARTS || GD == 0, "parts: one group per row");
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *const X = sm, *const B = sm + kDig * C::XB;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ int32_t mat_ex[kMaxD];
     __shared__ uint32_t next_tile[2];
-    __shared__ uint32_t part_max[GD ? 1 : C::TPR][kRows];
+    // largest parts: of a thread's amplitudes, or (PARTS) of each member
+    __shared__ uint32_t part_max[PARTS ? C::TPR * kSlots : GD ? 1 : C::TPR][kRows];
+    __shared__ int32_t row_odd[PARTS ? kRows : 1];
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int row = tid % kRows, part = tid / kRows;
@@ -376,16 +405,44 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
     I t = (I)blockIdx.x;
     if (t < ntiles) load(t, base);
     while (t < ntiles) {
-        int E[TG];
+        int E[PARTS ? kSlots : TG];  // of the inputs
+        uint32_t Eo[2] = {};         // PARTS: of the outputs, 16 bits each
         bool odd = false;
+        auto top_of = [](const double2 x) {
+            return max((uint32_t)__double2hiint(x.x) & 0x7fffffffu, (uint32_t)__double2hiint(x.y) & 0x7fffffffu);
+        };
+        // 1 (an exponent of 0) for parts whose leading words are zero and others not
+        auto tiny_of = [](const double2 x) { return (__double2loint(x.x) | __double2loint(x.y)) != 0 ? 1u : 0u; };
+        if constexpr (PARTS) {
+#pragma unroll
+            for (int c = 0; c < kSlots; ++c)
+                if (c < na) {
+                    const uint32_t top = top_of(v[c]);
+                    part_max[a0 + c][row] = top ? top : tiny_of(v[c]);
+                }
+            __syncthreads();
+            auto scale_of = [&](uint32_t m) {  // the mask is the same for a warp's lanes
+                uint32_t top = 0;
+                for (; m; m &= m - 1) top = max(top, part_max[__ffs((int)m) - 1][row]);
+                const int e = top ? scale_ex(top) : 1023;
+                odd = odd || e < kRowExLow || e > kRowExHigh;
+                return e;
+            };
+#pragma unroll
+            for (int c = 0; c < kSlots; ++c) {
+                E[c] = 1023;
+                if (c < na) {
+                    const uint32_t in = pt.in[a0 + c], out = pt.out[a0 + c];
+                    E[c] = scale_of(in);
+                    Eo[c / 2] |= (uint32_t)(out == in ? E[c] : scale_of(out)) << (c % 2 * 16);
+                }
+            }
+        } else
 #pragma unroll
         for (int k = 0; k < TG; ++k) {
             uint32_t top = 0;
 #pragma unroll
-            for (int u = 0; u < GS; ++u) {
-                const double2 x = v[k * GS + u];
-                top = max(top, max((uint32_t)__double2hiint(x.x) & 0x7fffffffu, (uint32_t)__double2hiint(x.y) & 0x7fffffffu));
-            }
+            for (int u = 0; u < GS; ++u) top = max(top, top_of(v[k * GS + u]));
             if constexpr (GD == 0) {
                 part_max[part][row] = top;
                 __syncthreads();
@@ -403,7 +460,8 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
 #pragma unroll
             for (int c = 0; c < kSlots; ++c) {
                 if (c < TG * GS && c < na) {
-                    to_digits(to_fields(v[c].x, E[c / GS]), to_fields(v[c].y, E[c / GS]), w[c]);
+                    const int e = E[PARTS ? c : c / GS];
+                    to_digits(to_fields(v[c].x, e), to_fields(v[c].y, e), w[c]);
                 } else {
 #pragma unroll
                     for (int s = 0; s < kDig; ++s) w[c][s] = 0u;
@@ -422,6 +480,13 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
         if (__syncthreads_or(odd || dead)) {  // rare: both reasons told apart by a second vote
             if (__syncthreads_or(dead)) break;
             any_odd = true;
+            if constexpr (PARTS) {  // the whole row, whichever part it was
+                if (part == 0) row_odd[row] = 0;
+                __syncthreads();
+                if (odd) row_odd[row] = 1;
+                __syncthreads();
+                odd = row_odd[row] != 0;
+            }
         }
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -463,7 +528,7 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
                     for (int l = 0; l < kLev; ++l) tmem_ld2_nowait(lane + (uint32_t)(l * C::K + 2 * c), acc[l]);
                     tmem_wait_ld();
                     const int k = c / GS, j = S::member(c, a0);
-                    const int e = E[k] + mat_ex[j] - 2044 - C::GRID;
+                    const int e = (PARTS ? (int)(Eo[c / 2] >> (c % 2 * 16) & 0xffffu) : E[k]) + mat_ex[j] - 2044 - C::GRID;
                     if (S::group(t, row, part, k) < a.R && !odd) {
                         const int64_t yr = sum_levels<C::GRID>(&acc[0][0], 2), yi = sum_levels<C::GRID>(&acc[0][1], 2);
                         if constexpr (TAB)
@@ -507,8 +572,8 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
     }
 }
 
-template <typename I, int NP, int GD, bool TAB>
-cudaError_t launch_tab(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+template <typename I, int NP, int GD, bool TAB, bool PARTS>
+cudaError_t launch_tab(const GatePlan &g, const TcCouples &tc, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
     using C = Tc64Cfg<NP, GD>;
     Tc64Args<I> a;
     a.psi = static_cast<double2 *>(psi);
@@ -541,7 +606,13 @@ cudaError_t launch_tab(const GatePlan &g, void *psi, int sm_count, int32_t *err,
     }
     for (int j = 0; j < kMaxD; ++j) a.off[j] = j < g.D ? (I)g.off[j] : 0;
     for (int k = 0; k < g.D * g.D; ++k) a.U[k] = make_double2(g.U[2 * k], g.U[2 * k + 1]);
-    auto fn = k_dense_tc64<I, NP, GD, TAB>;
+    Tc64Parts<PARTS> pt;
+    if constexpr (PARTS)
+        for (int j = 0; j < kMaxD; ++j) {
+            pt.in[j] = j < g.D ? tc.of_col[j] : 0u;
+            pt.out[j] = j < g.D ? tc.of_row[j] : 0u;
+        }
+    auto fn = k_dense_tc64<I, NP, GD, TAB, PARTS>;
     // 4 / NP CTAs on an SM, by their threads and the TMEM; the default split of
     // the L1 memory held one CTA less
     cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::DATA);
@@ -551,31 +622,80 @@ cudaError_t launch_tab(const GatePlan &g, void *psi, int sm_count, int32_t *err,
     const uint64_t tiles = (g.R + C::PER_TILE - 1) / C::PER_TILE;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * C::PER_SM);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, kChainL2Bytes, a, tb);
+    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, kChainL2Bytes, a, tb, pt);
 }
 
-template <typename I, int NP, int GD>
-cudaError_t launch_np(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+template <typename I, int NP, int GD, bool PARTS>
+cudaError_t launch_np(const GatePlan &g, const TcCouples &tc, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
     if constexpr (NP <= 2)
-        if (g.tab) return launch_tab<I, NP, GD, true>(g, psi, sm_count, err, s);
-    return launch_tab<I, NP, GD, false>(g, psi, sm_count, err, s);
+        if (g.tab) return launch_tab<I, NP, GD, true, PARTS>(g, tc, psi, sm_count, err, s);
+    return launch_tab<I, NP, GD, false, PARTS>(g, tc, psi, sm_count, err, s);
+}
+
+template <typename I, bool PARTS>
+cudaError_t launch_rows(const GatePlan &g, const TcCouples &tc, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+    if (g.D <= 8) return launch_np<I, 1, 0, PARTS>(g, tc, psi, sm_count, err, s);
+    if (g.D <= 16) return launch_np<I, 2, 0, PARTS>(g, tc, psi, sm_count, err, s);
+    if (g.D <= 24) return launch_np<I, 3, 0, PARTS>(g, tc, psi, sm_count, err, s);
+    return launch_np<I, 4, 0, PARTS>(g, tc, psi, sm_count, err, s);
 }
 
 template <typename I>
 cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+    TcCouples tc;
+    tc_couples(g.U.data(), g.D, kMatSpread, tc);
+    if (!tc.one) return launch_rows<I, true>(g, tc, psi, sm_count, err, s);
     switch (g.D) {
-        case 2: return launch_np<I, 1, 2>(g, psi, sm_count, err, s);
-        case 3: return launch_np<I, 1, 3>(g, psi, sm_count, err, s);
-        case 4: return launch_np<I, 1, 4>(g, psi, sm_count, err, s);
-        default: break;
+        case 2: return launch_np<I, 1, 2, false>(g, tc, psi, sm_count, err, s);
+        case 3: return launch_np<I, 1, 3, false>(g, tc, psi, sm_count, err, s);
+        case 4: return launch_np<I, 1, 4, false>(g, tc, psi, sm_count, err, s);
+        default: return launch_rows<I, false>(g, tc, psi, sm_count, err, s);
     }
-    if (g.D <= 8) return launch_np<I, 1, 0>(g, psi, sm_count, err, s);
-    if (g.D <= 16) return launch_np<I, 2, 0>(g, psi, sm_count, err, s);
-    if (g.D <= 24) return launch_np<I, 3, 0>(g, psi, sm_count, err, s);
-    return launch_np<I, 4, 0>(g, psi, sm_count, err, s);
 }
 
 }  // namespace
+
+bool tc_couples(const double *U, int D, int spread, TcCouples &c) {
+    const uint32_t all = D >= 32 ? ~0u : (1u << D) - 1u;
+    uint32_t part[kMaxD];
+    int n = 0;
+    c.one = true;
+    for (int j = 0; j < D; ++j) c.of_col[j] = 1u << j;
+    for (int i = 0; i < D; ++i) {
+        uint32_t m = 0;
+        int top = 0, low = 0x7ff;
+        for (int j = 0; j < D; ++j) {
+            const double re = std::fabs(U[2 * (i * D + j)]), im = std::fabs(U[2 * (i * D + j) + 1]);
+            if (re == 0.0 && im == 0.0) continue;
+            uint64_t a, b;
+            std::memcpy(&a, &re, 8);
+            std::memcpy(&b, &im, 8);
+            const int e = (int)(std::max(a, b) >> 52);
+            top = std::max(top, e);
+            low = std::min(low, e);
+            m |= 1u << j;
+        }
+        c.of_row[i] = m;
+        if (!m) continue;
+        if (top - low > spread) return false;
+        if (m != all) c.one = false;
+        bool known = false;
+        for (int k = 0; k < n; ++k) {
+            if (part[k] == m) known = true;
+            else if (part[k] & m) return false;
+        }
+        if (known) continue;
+        part[n++] = m;
+        for (int j = 0; j < D; ++j)
+            if (m >> j & 1u) c.of_col[j] = m;
+    }
+    return true;
+}
+
+bool tc64_matrix(const double *U, int D) {
+    TcCouples c;
+    return tc_matrix_ordinary(U, D, kMatExLow, kMatExHigh) && tc_couples(U, D, kMatSpread, c);
+}
 
 bool tc64_takes(const GatePlan &g) {
     if (g.kind != Kind::Dense || g.mode != Mode::Direct || g.D < 2 || g.D > (g.tab ? 16 : kMaxD)) return false;
@@ -586,7 +706,7 @@ bool tc64_takes(const GatePlan &g) {
     const double amps = (double)g.R * g.D;
     if (g.D == 2 && amps < 300000) return false;
     if (g.D == 3 && amps < 180000) return false;
-    return tc_matrix_ordinary(g, kMatExLow, kMatExHigh);
+    return tc64_matrix(g.U.data(), g.D);
 }
 
 cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
