@@ -163,5 +163,20 @@ def test_special_values_in_one_part(a, b):
     with np.errstate(all="ignore"):
         want = apply_ref(psi, dims, m, targets)
     most = allowed(m, np.where(fine, psi, 0), group, loc, L.QD_C128) + 2 * a * b * 2.0 ** -1074
-    assert np.all(np.abs((got - want).astype(np.complex128))[fine] <= most[fine])
+    assert np.all(np.abs((got[fine] - want[fine]).astype(np.complex128)) <= most[fine])
     assert not np.any(np.isfinite(got.real[~fine]) & np.isfinite(got.imag[~fine]))
+
+
+@pytest.mark.parametrize("d,dims", [(2, [2, 5, 61, 61, 17]), (3, [3, 61, 61, 17]), (4, [4] + OTHERS), (9, [9] + OTHERS), (27, [27] + OTHERS)])
+def test_groups_of_denormal_numbers(d, dims):
+    rng = np.random.default_rng(d)
+    psi = (rng.integers(-2000, 2000, math.prod(dims)) + 1j * rng.integers(-2000, 2000, math.prod(dims))) * 2.0 ** -1074
+    m = wl.haar_unitary(d, rng)
+    with L.Register(dims, None, L.QD_C128) as r:
+        L.qd_set_amplitudes(r.h, psi)
+        L.qd_apply(r.h, m, [0])
+        L.qd_sync(r.h)
+        got = r.amplitudes()
+    # every product is rounded to a multiple of 2^-1074: 2 D multiply-adds a part, half a unit each
+    err = np.abs((got - apply_ref(psi, dims, m, [0])).astype(np.clongdouble))
+    assert np.max(err) <= 2 * d * np.longdouble(2) ** -1074
