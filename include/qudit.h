@@ -139,7 +139,8 @@ int qd_set_stream(qd_reg *reg, void *stream);
  * >= 9; a value in 9..65 sends blocks of D >= value to the tensor cores
  * (exact products of short digits with FP32 accumulation) and smaller ones,
  * and single dense gates below it, to the CUDA-core dense kernels.  With the
- * default, dense launches of 10 to 16 states run on the tensor cores.  Blocks
+ * default, dense launches of 10 to 16 states whose matrix has no zeros (see
+ * qd_apply) run on the tensor cores.  Blocks
  * above 32 always run there, and complex128 dense launches from 4 states on
  * (2 and 3 on larger registers; for the matrices see qd_apply) whatever the
  * value. */
@@ -167,7 +168,13 @@ int qd_set_tuning(qd_reg *reg, int32_t key, int64_t value);
  * 2^10 of each other); output i is then off by at most
  * 4 D 2^-53 max_j |u_ij| max_j |v_j|, the maxima over the members j that row i
  * couples.  Other matrices are sums of rounded products, off by at most
- * 4 D 2^-53 sum_j |u_ij| |v_j|. */
+ * 4 D 2^-53 sum_j |u_ij| |v_j|.
+ * Complex64: matrices of 10 to 16 states without zeros (a row's entries within
+ * 2^8, the rows' largest within 2^3) run on the tensor cores, off by at most
+ * 4 D 2^-24 max |u| max_j |v_j|; all others are sums of rounded products, off
+ * by at most 6 D 2^-24 sum_j |u_ij| |v_j|.  Fused blocks in the tensor-core
+ * form (QD_FORM_BLOCK_TC) are off relative to the largest member whatever
+ * their matrix. */
 int qd_apply(qd_reg *reg, const double *matrix, const int32_t *targets, int32_t k,
              const int32_t *controls, const int32_t *ctrl_levels, int32_t nc);
 

@@ -14,6 +14,15 @@
 // rounding at the output's last place.  Dropped are products below 2^-35 of
 // the scale.
 //
+// An output's error is thus relative to the largest member of its group (and
+// the largest matrix entry), as in the BF16 kernel of qd_tc.cu, whose blocks
+// of up to 16 states this one took over.  The CUDA cores' is relative to the
+// output's own terms, so of the launches that would run there only those come
+// here whose matrix couples all members with entries of like size.  A gate on
+// one qudit of a 16-state pair, controlled or not, stays there: 334 against
+// 217 us below, but a half at 1e-9 of the other keeps its 24 bits (it became
+// zero on a common scale).
+//
 // A tile is 128 rows of 16 amplitude slots (K = 32), one group of D amplitudes
 // per row, spread evenly over its two threads.  The matrix digits are stacked
 // along N, so that digit s of the amplitudes meets all its partners in one MMA
@@ -63,6 +72,12 @@ constexpr int kRowExLow = 40, kRowExHigh = 210;
 // ... and (FP64 bias) of the matrix' largest entry, and how far below it that
 // of a row may lie (checked on the host; 28 bits of the row are left).
 constexpr int kMatExLow = 1023 - 20, kMatExHigh = 1023 + 20, kMatRows = 8;
+// Single gates and blocks priced on the CUDA cores, which round every product
+// to 24 bits of its own: every entry of the matrix must couple (no zeros, a
+// row's entries within 2^8), so that no output is small but by cancellation,
+// and rows lie within 2^3 of the largest entry (33 bits of each are left;
+// a unitary matrix' rows do).
+constexpr int kGateRows = 3, kGateSpread = 8;
 
 template <typename I>
 struct Tc32Args {
@@ -456,7 +471,10 @@ bool tc32_takes(const GatePlan &g, bool block, int sm_count) {
         if (consecutive) return false;
     }
     const int top = matrix_top(g);
-    return top >= kMatExLow && top <= kMatExHigh && tc_matrix_ordinary(g.U.data(), g.D, top - kMatRows, top);
+    if (top < kMatExLow || top > kMatExHigh) return false;
+    if (block) return tc_matrix_ordinary(g.U.data(), g.D, top - kMatRows, top);
+    TcCouples c;
+    return tc_matrix_ordinary(g.U.data(), g.D, top - kGateRows, top) && tc_couples(g.U.data(), g.D, kGateSpread, c) && c.one;
 }
 
 cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
