@@ -215,10 +215,8 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     // feature 11: log2 of the control-slice fraction, or (dense + table) of the table entries
     const double touched = dense_table ? (double)reg.N : (double)reg.N * std::exp2((double)lf.f[11]);
     const double b = c128 ? 16.0 : 8.0;
-    // 5.4 TB/s: what the memory-bound dense and mono kernels move on large
-    // registers (with 5.0 for mono a 2^32 Fourier ladder took a dense D = 16
-    // launch of 13.0 ms for a mono one of 5.9: 239.7 -> 244.8 ms)
-    double t_mem = 2.0 * touched * b / (table ? 5.0e12 : 5.4e12);
+    // complex128: 5.4 TB/s, what the memory-bound mono kernels move on large registers
+    double t_mem = 2.0 * touched * b / (c128 && !table ? 5.4e12 : 5.0e12);
     if (table) t_mem += std::exp2((double)lf.f[0]) * 16.0 / 5.0e12;
     if (dense_table) t_mem += std::exp2((double)lf.f[11]) * 16.0 / 5.0e12;
     // complex128 dense kernels: the CUDA cores take 4 D DFMA per amplitude; the
@@ -233,28 +231,25 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
         if (!lf.fp64) t_c128 = std::min(t_c128, t_tc);
     }
     double t_cmp = table ? touched * 40.0 / 2.0e13 : 0.0;  // index arithmetic per amplitude
-    if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : D <= 4.5 ? 0.0 : touched * (8.0 * D + 64.0) / 2.0e13;
+    if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : touched * (8.0 * D + 64.0) / 2.0e13;
     if (dense && !table && !dense_table) {
         if (!c128 && block) {
-            // fused block on the tensor cores: measured on GB300 it moves about
-            // 5.3 TB/s at D = Dp (5.1 up to 24, 4.95 above 32), less in proportion
-            // to the padding; up to D = 16 (qd_tc32.cu) 5.4 TB/s at full rows of 16 slots
+            // fused block on the tensor cores: 3.5 TB/s at D = Dp, less in proportion
+            // to the padding.  It moves 4.9 to 5.3 TB/s on large registers at strides
+            // of some amplitudes, but 3.3 on the lowest qudits (D = 27: 2.8), and on
+            // states that fit L2 it takes twice the CUDA-core launches' time; the
+            // features that a price is made of here do not tell these apart, and
+            // with 5.3 qutrit circuits were fused into D = 27 blocks at a loss (15
+            // qutrits, 41 gates, greedy 852 -> 1059 us; 14, exhaustive 87 -> 105)
             const double Dp = D <= 32 ? std::ceil(D / 8.0) * 8.0 : std::ceil(D / 16.0) * 16.0;
-            t_cmp = D < 16.5 ? touched * 4.7e-11 / D : 2.0 * touched * b / ((D <= 24.5 ? 5.1e12 : D <= 32.5 ? 5.3e12 : 4.95e12) * D / Dp);
+            t_cmp = 2.0 * touched * b / (3.5e12 * D / Dp);
         } else {
-            // complex64 with hi+lo coefficients: hidden under the memory pass up to
-            // D = 8, then 8 D FFMA per amplitude plus index work (packed at D = 9);
-            // from D = 10 to 16 the tensor cores (qd_tc32.cu) at rows of 16 slots
-            t_cmp = c128 ? t_c128 : D < 8.5 ? 0.0 : touched * (8.0 * D + 24.0) / (D < 9.5 ? 2.4e13 : 2.0e13);
-            if (!c128 && D > 9.5 && D < 16.5) t_cmp = std::min(t_cmp, touched * 4.7e-11 / D);
+            // complex64 with hi+lo coefficients: 8 D FFMA per amplitude plus
+            // index work
+            t_cmp = c128 ? t_c128 : touched * (8.0 * D + 24.0) / 2.0e13;
         }
     }
-    // a launch, and what the complex64 dense kernels take longer than a mono
-    // kernel on a state of a few amplitudes (1.5 us: 0.1 at D = 4, 0.6 at D = 8,
-    // 2.0 to 2.5 from D = 9 on): without it a plan of a small register takes a
-    // dense launch where a mono one is as good
-    const double setup = !dense || c128 ? 0.0 : D < 8.5 ? 0.07e-6 * D : 2.0e-6;
-    return std::max(t_mem, t_cmp) + setup + 4.0e-6;
+    return std::max(t_mem, t_cmp) + 4.0e-6;
 }
 
 double segment_cost(const std::vector<FuseGate> &gates, int first, int last, const RegisterShape &reg,
