@@ -594,6 +594,7 @@ static int smem_bytes_for(int Dp) {
 }
 
 int tc_smem_bytes(int Dp) {
+    if (Dp <= 16) return smem_bytes_for<16>(Dp);
     if (Dp <= 32) return smem_bytes_for<32>(Dp);
     return smem_bytes_for<64>(Dp);
 }
@@ -631,6 +632,8 @@ static cudaError_t launch_tc_im(const GatePlan &g, void *psi, int sm_count, int3
 
 template <typename I>
 static cudaError_t launch_tc_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+    // up to 16 states: the blocks whose matrix qd_tc32.cu does not take
+    if (g.Dp <= 16) return launch_tc_im<I, 16>(g, psi, sm_count, err, s);
     if (g.Dp <= 32) return launch_tc_im<I, 32>(g, psi, sm_count, err, s);
     return launch_tc_im<I, 64>(g, psi, sm_count, err, s);
 }

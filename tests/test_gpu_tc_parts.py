@@ -213,3 +213,69 @@ def test_norm_after_many_gates_of_16_states():
         r.run(gates, L.QD_PLAN_NONE)
         after = L.qd_norm(r.h)
     assert abs(after - before) <= 3e-8
+
+
+def unusual(kind, d, rng, prec):
+    """Matrices outside the exponents that the digits of qd_tc32.cu and qd_tc64.cu hold."""
+    m = wl.haar_unitary(d, rng)
+    far = 30 if prec == L.QD_C64 else 150
+    if kind == "small":
+        return m * 2.0 ** -far
+    if kind == "large":
+        return m * 2.0 ** far
+    m[1] *= 2.0 ** (-12 if prec == L.QD_C64 else -far)
+    return m
+
+
+@pytest.mark.parametrize("kind", ["small", "large", "one row"])
+@pytest.mark.parametrize("dims", [[3, 3], [4, 3], [2, 7], [4, 4]], ids=str)
+def test_blocks_of_unusual_matrices(dims, kind):
+    """Tensor-core blocks of 9 to 16 states that run on the kernel of the larger ones: parts in three BF16
+    slices, 2^-27 of a scale of at most 2 V (the group's largest), rows likewise of 2 R, and three
+    roundings of at most D R V: below D 2^-22 R V for every row."""
+    rng = np.random.default_rng(2)
+    d = math.prod(dims)
+    regs, targets = dims + OTHERS, [1, 0]
+    first = wl.haar_unitary(d, rng)
+    m = unusual(kind, d, rng, L.QD_C64)
+    gates = [wl.Gate("U", tuple(targets), matrix=first), wl.Gate("U", tuple(targets), matrix=m @ first.conj().T)]
+    group, loc = members(regs, targets)
+    psi = (rng.standard_normal(group.size) + 1j * rng.standard_normal(group.size)).astype(np.complex64)
+    for index64 in (0, 1):
+        with L.Register(regs, None, L.QD_C64) as r:
+            L.qd_set_tuning(r.h, L.QD_TUNE_INDEX64, index64)
+            L.qd_set_amplitudes(r.h, psi)
+            plan = L.qd_plan_create_forms(r.h, gates, [(0, 1)], [L.QD_FORM_BLOCK_TC])
+            L.qd_plan_run(plan)
+            L.qd_sync(r.h)
+            got = r.amplitudes()
+            L.qd_plan_destroy(plan)
+        err = np.abs((got - apply_ref(psi, regs, m, targets)).astype(complex))
+        v = np.zeros(group.max() + 1)
+        np.maximum.at(v, group, np.abs(psi))
+        assert np.all(err <= d * 2.0 ** -22 * v[group] * np.abs(m).max(axis=1)[loc])
+
+
+@pytest.mark.parametrize("prec", [L.QD_C64, L.QD_C128])
+@pytest.mark.parametrize("kind", ["small", "large", "one row"])
+@pytest.mark.parametrize("d", [4, 9, 12, 16, 27])
+def test_gates_of_unusual_matrices(d, kind, prec):
+    rng = np.random.default_rng(d)
+    m = unusual(kind, d, rng, prec)
+    dims = [7, d, 61, 5]
+    group, loc = members(dims, [1])
+    psi = (rng.standard_normal(group.size) + 1j * rng.standard_normal(group.size)).astype(DTYPE[prec])
+    check(prec, dims, [1], m, psi)
+    if prec == L.QD_C128 and d <= 16:  # with a run: the table of a phase per level of qudit 0
+        phases = np.exp(2j * np.pi * rng.random(7))
+        gates = [wl.Gate("U", (1,), matrix=m), wl.Gate("DIAG", (0,), matrix=phases)]
+        with L.Register(dims, None, prec) as r:
+            L.qd_set_amplitudes(r.h, psi)
+            plan = L.qd_plan_create_forms(r.h, gates, [(0, 1)], [L.QD_FORM_DENSE_RUN])
+            L.qd_plan_run(plan)
+            L.qd_sync(r.h)
+            got = r.amplitudes()
+            L.qd_plan_destroy(plan)
+        want = apply_ref(psi, dims, m, [1]) * phases[np.arange(group.size) % 7]
+        most = allowed(m, psi, group, loc, prec) + 4 * 2.0 ** -53 * np.abs(want.astype(complex))
+        assert np.all(np.abs((got - want).astype(np.complex128)) <= most)
