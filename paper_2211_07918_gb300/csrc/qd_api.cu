@@ -884,9 +884,10 @@ bool has_measure(const qd_gate *gates, int32_t ngates) {
 }
 
 // Validate every gate, drop identities, and collect both the fusion view
-// (matrix over controls + targets) and the original records.
+// (matrix over controls + targets) and the original records.  priced: the
+// segments will be priced (what only a price needs is left out otherwise).
 int collect_gates(const qd_reg *r, const qd_gate *gates, int32_t ngates, std::vector<FuseGate> &fg,
-                  std::vector<const qd_gate *> &orig) {
+                  std::vector<const qd_gate *> &orig, bool priced = true) {
     for (int i = 0; i < ngates; ++i) {
         const qd_gate *gt = &gates[i];
         if (gt->kind == QD_GATE_MEASURE) break;  // gates after the measurement flag are ignored (Sec. 3.4)
@@ -913,7 +914,7 @@ int collect_gates(const qd_reg *r, const qd_gate *gates, int32_t ngates, std::ve
                 bool ident = g.kind == Kind::Mono;  // a permutation with phases whose permutation is the identity
                 for (int j = 0; ident && j < a.D; ++j) ident = g.src[j] == j;
                 fg.back().diag = ident;
-                fg.back().fp64 = r->prec == QD_C128 && g.kind == Kind::Dense && !tc64_matrix(g.U.data(), g.D);
+                fg.back().fp64 = priced && r->prec == QD_C128 && g.kind == Kind::Dense && !tc64_matrix(g.U.data(), g.D);
                 orig.push_back(gt);
             }
         }
@@ -1274,7 +1275,7 @@ int qd_plan_create(qd_reg *r, const qd_gate *gates, int32_t ngates, int32_t plan
     if (plan_kind < QD_PLAN_NONE || plan_kind > QD_PLAN_EXHAUSTIVE) return fail(QD_ERR_ARG, "unknown plan kind");
     std::vector<FuseGate> fg;
     std::vector<const qd_gate *> orig;
-    int rc = collect_gates(r, gates, ngates, fg, orig);
+    int rc = collect_gates(r, gates, ngates, fg, orig, plan_kind != QD_PLAN_NONE);
     if (rc) return rc;
     std::vector<std::pair<int, int>> segs;
     std::vector<int> kinds;

@@ -317,7 +317,6 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
     constexpr int TG = C::TG;
     constexpr int GS = GD ? GD : kSlots;  // slots of a group in this thread
     constexpr bool QUEUE = GD != 0;
-    static_assert(!PARTS || GD == 0, "parts: one group per row");
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *const X = sm, *const B = sm + kDig * C::XB;
     __shared__ uint32_t tmem_base;
@@ -325,8 +324,8 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
     __shared__ int32_t mat_ex[kMaxD];
     __shared__ uint32_t next_tile[2];
     // largest parts: of a thread's amplitudes, or (PARTS) of each member
-    __shared__ uint32_t part_max[PARTS ? C::TPR * kSlots : GD ? 1 : C::TPR][kRows];
-    __shared__ int32_t row_odd[PARTS ? kRows : 1];
+    __shared__ uint32_t part_max[GD ? 1 : PARTS ? C::TPR * kSlots : C::TPR][kRows];
+    __shared__ int32_t row_odd[PARTS && !GD ? kRows : 1];
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int row = tid % kRows, part = tid / kRows;
@@ -413,7 +412,26 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
         };
         // 1 (an exponent of 0) for parts whose leading words are zero and others not
         auto tiny_of = [](const double2 x) { return (__double2loint(x.x) | __double2loint(x.y)) != 0 ? 1u : 0u; };
-        if constexpr (PARTS) {
+        if constexpr (PARTS && GD) {  // whole groups in this thread
+            uint32_t top[kSlots];
+#pragma unroll
+            for (int c = 0; c < TG * GS; ++c) {
+                top[c] = top_of(v[c]);
+                top[c] = top[c] ? top[c] : tiny_of(v[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < TG * GS; ++c) {
+                uint32_t ti = 0, to = 0;
+#pragma unroll
+                for (int u = 0; u < GS; ++u) {
+                    if (pt.in[c % GS] >> u & 1u) ti = max(ti, top[c / GS * GS + u]);
+                    if (pt.out[c % GS] >> u & 1u) to = max(to, top[c / GS * GS + u]);
+                }
+                E[c] = ti ? scale_ex(ti) : 1023;
+                odd = odd || E[c] < kRowExLow || E[c] > kRowExHigh;
+                Eo[c / 2] |= (uint32_t)(to ? scale_ex(to) : 1023) << (c % 2 * 16);
+            }
+        } else if constexpr (PARTS) {
 #pragma unroll
             for (int c = 0; c < kSlots; ++c)
                 if (c < na) {
@@ -490,7 +508,7 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
         if (__syncthreads_or(odd || dead)) {  // rare: both reasons told apart by a second vote
             if (__syncthreads_or(dead)) break;
             any_odd = true;
-            if constexpr (PARTS) {  // the whole row, whichever part it was
+            if constexpr (PARTS && !GD) {  // the whole row, whichever part it was
                 if (part == 0) row_odd[row] = 0;
                 __syncthreads();
                 if (odd) row_odd[row] = 1;
@@ -654,7 +672,11 @@ template <typename I>
 cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
     TcCouples tc;
     tc_couples(g.U.data(), g.D, kMatSpread, tc);
-    if (!tc.one) return launch_rows<I, true>(g, tc, psi, sm_count, err, s);
+    if (!tc.one) switch (g.D) {
+        case 3: return launch_np<I, 1, 3, true>(g, tc, psi, sm_count, err, s);
+        case 4: return launch_np<I, 1, 4, true>(g, tc, psi, sm_count, err, s);
+        default: return launch_rows<I, true>(g, tc, psi, sm_count, err, s);
+    }
     switch (g.D) {
         case 2: return launch_np<I, 1, 2, false>(g, tc, psi, sm_count, err, s);
         case 3: return launch_np<I, 1, 3, false>(g, tc, psi, sm_count, err, s);

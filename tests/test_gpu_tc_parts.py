@@ -94,6 +94,19 @@ def test_parts_have_their_own_scale(a, b, kind, index64):
         check(L.QD_C128, dims, targets, m, state(m, group, loc, rng, L.QD_C128), index64)
 
 
+@pytest.mark.parametrize("index64", [0, 1])
+@pytest.mark.parametrize("dims,target", [([3, 61, 61, 17], 0), ([61, 3, 61, 17], 1), ([61, 61, 18, 3], 3)], ids=str)
+def test_parts_of_three_states(dims, target, index64):
+    """One state alone and two coupled, in place and moved, on registers that take the tensor cores."""
+    rng = np.random.default_rng(9)
+    m = np.eye(3, dtype=complex)
+    m[1:, 1:] = wl.haar_unitary(2, rng)
+    group, loc = members(dims, [target])
+    for p, q in (([0, 1, 2], [0, 1, 2]), ([2, 0, 1], [0, 2, 1]), ([1, 2, 0], [1, 0, 2])):
+        mm = m[p][:, q]
+        check(L.QD_C128, dims, [target], mm, state(mm, group, loc, rng, L.QD_C128), index64)
+
+
 @pytest.mark.parametrize("a,b", [(2, 5), (3, 4), (2, 7), (5, 3), (4, 4)])
 @pytest.mark.parametrize("kind", ["high alone", "low alone", "blocks", "controlled", "moved"])
 def test_parts_of_single_precision_gates(a, b, kind):
