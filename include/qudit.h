@@ -165,7 +165,7 @@ int qd_set_tuning(qd_reg *reg, int32_t key, int64_t value);
  * Accuracy of a complex128 dense matrix U on a group v of D amplitudes: the
  * tensor cores take matrices that fall into full parts (any two rows couple
  * the same members or none in common, a row's non-zero entries lie within
- * 2^10 of each other); output i is then off by at most
+ * 2^12 of each other); output i is then off by at most
  * 4 D 2^-53 max_j |u_ij| max_j |v_j|, the maxima over the members j that row i
  * couples.  Other matrices are sums of rounded products, off by at most
  * 4 D 2^-53 sum_j |u_ij| |v_j|.

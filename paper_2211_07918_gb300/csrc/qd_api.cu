@@ -157,7 +157,8 @@ cudaError_t launch_plan(const qd_reg *r, const GatePlan &g) {
         if (tc32_takes(g, false, r->sm_count)) return launch_dense_tc32(g, r->psi, r->sm_count, r->dev_err, r->stream);
         return launch_gate_f32(g, r->psi, r->sm_count, r->stream);
     }
-    if (tc64_takes(g)) return launch_dense_tc64(g, r->psi, r->sm_count, r->dev_err, r->stream);
+    TcCouples c;
+    if (tc64_takes(g, c)) return launch_dense_tc64(g, c, r->psi, r->sm_count, r->dev_err, r->stream);
     return launch_gate_f64(g, r->psi, r->sm_count, r->stream);
 }
 

@@ -23,14 +23,6 @@ int tc_smem_bytes(int Dp);
 // Launch one block (g.mode == Mode::Tensor) on a complex64 state.
 cudaError_t launch_block_tc(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
 
-// Dense gates and blocks of complex128 states (qd_tc64.cu): whether the kernel
-// takes a launch (direct geometry, matrix entries of ordinary size, for D < 4
-// enough amplitudes in the gate's slice), and the launch.  err: the
-// error word, followed by the queue words 2 and 3, zero between launches; the
-// launches that share it are ordered on one stream.
-bool tc64_takes(const GatePlan &g);
-cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s);
-
 // Dense gates and blocks of complex64 states of kTcMinD to 16 states
 // (qd_tc32.cu): whether the kernel takes a launch (direct geometry, matrix
 // entries of ordinary size; for a single gate or a block priced on the CUDA
@@ -49,13 +41,22 @@ struct TcCouples {
     uint32_t of_row[kMaxD], of_col[kMaxD];
 };
 // False where the parts are not told apart by the zeros of the rows (two rows
-// share some of their members, not all) or the exponents of a row's entries
-// differ by more than `spread`: an output may then be much smaller than the
+// share some of their members, not all), the exponents of a row's entries
+// differ by more than `spread`, or that of its largest part lies outside
+// [low_top, high_top].  An output may otherwise be much smaller than the
 // largest member of its part for other reasons than cancellation, and a scale
 // per part does not hold it to the accuracy of a sum of rounded products.
-bool tc_couples(const double *U, int D, int spread, TcCouples &c);
+bool tc_couples(const double *U, int D, int low_top, int high_top, int spread, TcCouples &c);
 
-// Whether k_dense_tc64 takes a launch with this matrix.
+// Dense gates and blocks of complex128 states (qd_tc64.cu): whether the kernel
+// takes a launch (direct geometry, a matrix of full parts with entries of
+// ordinary size, for D < 4 enough amplitudes in the gate's slice), with the
+// parts, and the launch.  err: the error word, followed by the queue words 2
+// and 3, zero between launches; the launches that share it are ordered on one
+// stream.
+bool tc64_takes(const GatePlan &g, TcCouples &c);
+cudaError_t launch_dense_tc64(const GatePlan &g, const TcCouples &c, void *psi, int sm_count, int32_t *err, cudaStream_t s);
+// Whether the matrix alone lets a launch be taken.
 bool tc64_matrix(const double *U, int D);
 
 }  // namespace qd

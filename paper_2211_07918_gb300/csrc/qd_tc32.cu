@@ -474,7 +474,7 @@ bool tc32_takes(const GatePlan &g, bool block, int sm_count) {
     if (top < kMatExLow || top > kMatExHigh) return false;
     if (block) return tc_matrix_ordinary(g.U.data(), g.D, top - kMatRows, top);
     TcCouples c;
-    return tc_matrix_ordinary(g.U.data(), g.D, top - kGateRows, top) && tc_couples(g.U.data(), g.D, kGateSpread, c) && c.one;
+    return tc_couples(g.U.data(), g.D, top - kGateRows, top, kGateSpread, c) && c.one;
 }
 
 cudaError_t launch_dense_tc32(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {

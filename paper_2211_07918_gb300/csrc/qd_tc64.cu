@@ -25,7 +25,7 @@
 // one: a matrix that falls into parts (a controlled gate or a gate on one of
 // its qudits, as a block; tc_couples) has a scale for each part of each group
 // (PARTS), and matrices whose rows share some of their members, or hold
-// entries more than 2^10 apart, stay on the FP64 pipe.  With a single scale,
+// entries more than 2^12 apart, stay on the FP64 pipe.  With a single scale,
 // the half of diag(R, R) at 1e-12 of the other was off by 1e-6 of itself; with
 // two by 4e-16.
 //
@@ -53,11 +53,10 @@
 // D = 32: 304 -> 14 us (one thread's serial chain of FP64 operations before).
 // Matrices of parts (a gate on the lower qudit; controlled), single scale ->
 // a scale per part (the loop over a part's members, uniform in a warp, and up
-// to two scales per amplitude): D = 4 278 -> 471; 457 (a group per row instead
-// of four; CUDA cores 1039), D = 9 413 -> 495; 463 (2321), D = 16 356 -> 449;
+// to two scales per amplitude): D = 4 278 -> 316 for both (CUDA cores 1039; 471
+// with a group per row instead of four), D = 9 413 -> 495; 463 (2321), D = 16 356 -> 449;
 // 416 (4113), D = 27 473 -> 618; 545 (8365).
 #include <algorithm>
-#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -84,7 +83,7 @@ constexpr int kRowExLow = 400, kRowExHigh = 1900;
 // ... and of a matrix row's largest entry (checked on the host).
 constexpr int kMatExLow = 923, kMatExHigh = 1123;
 // ... and how far below it the row's smallest non-zero entry may lie.
-constexpr int kMatSpread = 10;
+constexpr int kMatSpread = 12;
 
 template <typename I>
 struct Tc64Args {
@@ -669,9 +668,7 @@ cudaError_t launch_rows(const GatePlan &g, const TcCouples &tc, void *psi, int s
 }
 
 template <typename I>
-cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
-    TcCouples tc;
-    tc_couples(g.U.data(), g.D, kMatSpread, tc);
+cudaError_t launch_i(const GatePlan &g, const TcCouples &tc, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
     if (!tc.one) switch (g.D) {
         case 3: return launch_np<I, 1, 3, true>(g, tc, psi, sm_count, err, s);
         case 4: return launch_np<I, 1, 4, true>(g, tc, psi, sm_count, err, s);
@@ -687,7 +684,7 @@ cudaError_t launch_i(const GatePlan &g, void *psi, int sm_count, int32_t *err, c
 
 }  // namespace
 
-bool tc_couples(const double *U, int D, int spread, TcCouples &c) {
+bool tc_couples(const double *U, int D, int low_top, int high_top, int spread, TcCouples &c) {
     const uint32_t all = D >= 32 ? ~0u : (1u << D) - 1u;
     uint32_t part[kMaxD];
     int n = 0;
@@ -697,19 +694,18 @@ bool tc_couples(const double *U, int D, int spread, TcCouples &c) {
         uint32_t m = 0;
         int top = 0, low = 0x7ff;
         for (int j = 0; j < D; ++j) {
-            const double re = std::fabs(U[2 * (i * D + j)]), im = std::fabs(U[2 * (i * D + j) + 1]);
-            if (re == 0.0 && im == 0.0) continue;
-            uint64_t a, b;
-            std::memcpy(&a, &re, 8);
-            std::memcpy(&b, &im, 8);
-            const int e = (int)(std::max(a, b) >> 52);
+            uint64_t p[2];
+            std::memcpy(p, &U[2 * (i * D + j)], 16);
+            const uint64_t larger = std::max(p[0] & ~(1ull << 63), p[1] & ~(1ull << 63));
+            if (!larger) continue;
+            const int e = (int)(larger >> 52);
             top = std::max(top, e);
             low = std::min(low, e);
             m |= 1u << j;
         }
         c.of_row[i] = m;
         if (!m) continue;
-        if (top - low > spread) return false;
+        if (top < low_top || top > high_top || top - low > spread) return false;
         if (m != all) c.one = false;
         bool known = false;
         for (int k = 0; k < n; ++k) {
@@ -726,10 +722,10 @@ bool tc_couples(const double *U, int D, int spread, TcCouples &c) {
 
 bool tc64_matrix(const double *U, int D) {
     TcCouples c;
-    return tc_matrix_ordinary(U, D, kMatExLow, kMatExHigh) && tc_couples(U, D, kMatSpread, c);
+    return tc_couples(U, D, kMatExLow, kMatExHigh, kMatSpread, c);
 }
 
-bool tc64_takes(const GatePlan &g) {
+bool tc64_takes(const GatePlan &g, TcCouples &c) {
     if (g.kind != Kind::Dense || g.mode != Mode::Direct || g.D < 2 || g.D > (g.tab ? 16 : kMaxD)) return false;
     // 5 us of setup against a serial chain of 4 D FP64 multiply-adds per thread:
     // D = 2 6.2 against 6.7 us on 262,144 amplitudes, 19.2 against 12.6 on 2^20;
@@ -738,12 +734,12 @@ bool tc64_takes(const GatePlan &g) {
     const double amps = (double)g.R * g.D;
     if (g.D == 2 && amps < 300000) return false;
     if (g.D == 3 && amps < 180000) return false;
-    return tc64_matrix(g.U.data(), g.D);
+    return tc_couples(g.U.data(), g.D, kMatExLow, kMatExHigh, kMatSpread, c);
 }
 
-cudaError_t launch_dense_tc64(const GatePlan &g, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
-    if (!wide_index(g)) return launch_i<uint32_t>(g, psi, sm_count, err, s);
-    return launch_i<uint64_t>(g, psi, sm_count, err, s);
+cudaError_t launch_dense_tc64(const GatePlan &g, const TcCouples &c, void *psi, int sm_count, int32_t *err, cudaStream_t s) {
+    if (!wide_index(g)) return launch_i<uint32_t>(g, c, psi, sm_count, err, s);
+    return launch_i<uint64_t>(g, c, psi, sm_count, err, s);
 }
 
 }  // namespace qd
