@@ -649,7 +649,18 @@ cudaError_t launch_tab(const GatePlan &g, const TcCouples &tc, void *psi, int sm
     const uint64_t tiles = (g.R + C::PER_TILE - 1) / C::PER_TILE;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sm_count * C::PER_SM);
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, kChainL2Bytes, a, tb, pt);
+    // Not chained: launches of about a tile per SM where SMs hold several CTAs.
+    // The next launch's CTAs come early, some SMs get several of them and others
+    // none, and their tiles take longer than the launch latency that is gained.
+    // us per gate, unchained / chained, tiles in brackets, on 152 SMs.  Four CTAs
+    // an SM: D = 4 5.8 / 5.5 (64), 5.8 / 7.1 (128), 6.8 / 7.4 (256), 9.9 / 8.0 (512);
+    // D = 6 4.9 / 4.4 (64), 4.9 / 6.4 (128), 6.5 / 6.9 (256), 9.2 / 7.4 (512); D = 8
+    // 5.3 / 5.3 (64), 5.3 / 7.5 (128), 7.2 / 7.8 (256), 10.5 / 8.7 (512).  Two: D = 16
+    // 7.4 / 6.5 (16), 7.3 / 7.6 (32), 7.4 / 8.9 (64), 7.5 / 9.5 (128), 11.1 / 9.8 (256);
+    // D = 9 6.0 / 5.4 (52), 8.1 / 6.3 (154).  One: D = 27 13.1 / 11.4 (52).
+    const uint64_t sms = (uint64_t)sm_count;
+    const bool alone = NP == 1 ? tiles > sms / 2 && tiles <= 2 * sms : NP == 2 ? tiles > sms * 3 / 8 && tiles <= sms : false;
+    return launch_chained(fn, grid, C::THREADS, C::DATA, s, 16 * g.N, alone ? 0 : kChainL2Bytes, a, tb, pt);
 }
 
 template <typename I, int NP, int GD, bool PARTS>
