@@ -276,9 +276,10 @@ int qd_plan_destroy(qd_plan *plan);
 #define QD_KCLASS_DENSE_TILE 1
 #define QD_KCLASS_MONO_DIRECT 2
 #define QD_KCLASS_MONO_TILE 3
-#define QD_KCLASS_TENSOR_BLOCK 4 /* fused block on tcgen05 (exact BF16 slices, FP32 accumulate) */
+#define QD_KCLASS_TENSOR_BLOCK 4 /* complex64 fused block on tcgen05 (exact products of short digits, FP32 accumulate) */
 #define QD_KCLASS_DIAG_TABLE 5   /* run of diagonal gates through one table (D = qudits the table covers) */
 #define QD_KCLASS_DENSE_TABLE 6  /* dense part followed by a diagonal run's table, one pass (D = dense part) */
+#define QD_KCLASS_TC 0x80        /* with DENSE_DIRECT or DENSE_TABLE: the launch runs on the tensor cores */
 int qd_plan_profile(qd_plan *plan, int32_t enable);
 int qd_plan_timings(qd_plan *plan, float *ms, double *alg_bytes, int32_t *kclass);
 /* Plan, run once with direct launches (no graph capture) and release. */

@@ -1517,6 +1517,9 @@ int qd_plan_timings(qd_plan *p, float *ms, double *alg_bytes, int32_t *kclass) {
             if (g.mode == Mode::Tensor) c = QD_KCLASS_TENSOR_BLOCK;
             if (g.mode == Mode::Table) c = QD_KCLASS_DIAG_TABLE;
             if (g.mode == Mode::Direct && g.tab) c = QD_KCLASS_DENSE_TABLE;
+            TcCouples tc;  // as launch_plan chooses
+            if (g.mode == Mode::Direct && (p->reg->prec == QD_C64 ? tc32_takes(g, false, p->reg->sm_count) : tc64_takes(g, tc)))
+                c |= QD_KCLASS_TC;
             kclass[i] = c | (g.D << 8);
         }
     }

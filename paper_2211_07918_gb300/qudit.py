@@ -311,6 +311,7 @@ def qd_plan_profile(plan: int, enable: bool = True) -> None:
     _check(load().qd_plan_profile(_vp(plan), 1 if enable else 0))
 
 
+QD_KCLASS_TC = 0x80
 KCLASS_NAMES = {0: "dense_direct", 1: "dense_tile", 2: "mono_direct", 3: "mono_tile", 4: "tensor_block",
                 5: "diag_table", 6: "dense_table"}
 
@@ -327,7 +328,7 @@ def qd_plan_timings(plan: int, with_times: bool = True):
 
 
 def kclass_name(c: int) -> str:
-    return f"{KCLASS_NAMES[c & 0xff]}_D{c >> 8}"
+    return f"{KCLASS_NAMES[c & 0x7f]}_D{c >> 8}" + ("_tc" if c & QD_KCLASS_TC else "")
 
 
 def qd_plan_destroy(plan: int) -> None:
