@@ -170,7 +170,7 @@ int qd_set_tuning(qd_reg *reg, int32_t key, int64_t value);
  * couples.  Other matrices are sums of rounded products, off by at most
  * 4 D 2^-53 sum_j |u_ij| |v_j|.
  * Complex64: matrices of 10 to 16 states without zeros (a row's entries within
- * 2^8, the rows' largest within 2^3) run on the tensor cores, off by at most
+ * 2^10, the rows' largest within 2^3) run on the tensor cores, off by at most
  * 4 D 2^-24 max |u| max_j |v_j|; all others are sums of rounded products, off
  * by at most 6 D 2^-24 sum_j |u_ij| |v_j|.  Fused blocks in the tensor-core
  * form (QD_FORM_BLOCK_TC) are off relative to the largest member whatever

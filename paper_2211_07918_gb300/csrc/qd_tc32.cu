@@ -40,7 +40,9 @@
 // (330 against 373 us: a thread's eight lie in a line of their own).  Up to
 // D = 8 the CUDA cores are not the limit (5.4 to 6.3 TB/s against 4.5 to 5.4),
 // above D = 16 the warp-specialised kernel is as fast or faster (D = 18 3.87
-// TB/s both, D = 27 4.24 against 3.82).
+// TB/s both, D = 27 4.24 against 3.82).  64-bit indices, CUDA cores -> here:
+// D = 10 on 8.8e9 amplitudes 49.1 -> 46.7 ms, D = 13 47.3 -> 41.1, D = 16 (8.5e9)
+// 44.2 -> 37.0 (42 bytes spilled).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -74,10 +76,10 @@ constexpr int kRowExLow = 40, kRowExHigh = 210;
 constexpr int kMatExLow = 1023 - 20, kMatExHigh = 1023 + 20, kMatRows = 8;
 // Single gates and blocks priced on the CUDA cores, which round every product
 // to 24 bits of its own: every entry of the matrix must couple (no zeros, a
-// row's entries within 2^8), so that no output is small but by cancellation,
+// row's entries within 2^10), so that no output is small but by cancellation,
 // and rows lie within 2^3 of the largest entry (33 bits of each are left;
 // a unitary matrix' rows do).
-constexpr int kGateRows = 3, kGateSpread = 8;
+constexpr int kGateRows = 3, kGateSpread = 10;
 
 template <typename I>
 struct Tc32Args {
