@@ -53,9 +53,13 @@
 // D = 32: 304 -> 14 us (one thread's serial chain of FP64 operations before).
 // Matrices of parts (a gate on the lower qudit; controlled), single scale ->
 // a scale per part (the loop over a part's members, uniform in a warp, and up
-// to two scales per amplitude): D = 4 278 -> 316 for both (CUDA cores 1039; 471
-// with a group per row instead of four), D = 9 413 -> 495; 463 (2321), D = 16 356 -> 449;
-// 416 (4113), D = 27 473 -> 618; 545 (8365).
+// to two scales per amplitude): D = 4 278 -> 314 for both (471 with a group per
+// row instead of four; CUDA cores 1039), D = 9 413 -> 464; 461 (2321), D = 16
+// 356 -> 412; 415 (4113), D = 27 473 -> 526; 524 (8365; 618 for the first with a
+// loop for every member).
+// 64-bit indices, on the FP64 pipe -> here: D = 3 on 2.6e9 amplitudes 58.9 ->
+// 22.0 ms, D = 9 on 2.4e9 163 -> 40, D = 27 586 -> 40 (the kernels hold their
+// bases in twice the registers and spill up to 122 bytes).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -450,7 +454,8 @@ __global__ void __launch_bounds__(Tc64Cfg<NP, GD>::THREADS, Tc64Cfg<NP, GD>::PER
                 E[c] = 1023;
                 if (c < na) {
                     const uint32_t in = pt.in[a0 + c], out = pt.out[a0 + c];
-                    E[c] = scale_of(in);
+                    // (a gate on the lower qudits of a block: neighbours are of one part)
+                    E[c] = c && in == pt.in[a0 + c - (c ? 1 : 0)] ? E[c ? c - 1 : 0] : scale_of(in);
                     Eo[c / 2] |= (uint32_t)(out == in ? E[c] : scale_of(out)) << (c % 2 * 16);
                 }
             }
