@@ -228,7 +228,9 @@ double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     if (c128) {
         const double Dp = std::ceil(D / 8.0) * 8.0;
         const double t_tc = touched * (D <= 4.5 ? 8.2e-12 : D <= 16.5 ? 9.6e-12 * (1.0 + 0.65 * (Dp - D) / Dp) : 15.0e-12) + 1.0e-6;
-        if (!lf.fp64) t_c128 = std::min(t_c128, t_tc);
+        // on the FP64 pipe a thread's 4 D^2 dependent multiply-adds are the least
+        // a launch takes (D = 4 6, D = 9 25, D = 16 78, D = 27 258, D = 32 305 us)
+        t_c128 = lf.fp64 ? std::max(t_c128, 0.31e-6 * D * D) : std::min(t_c128, t_tc);
     }
     double t_cmp = table ? touched * 40.0 / 2.0e13 : 0.0;  // index arithmetic per amplitude
     if (dense_table) t_cmp = c128 ? t_c128 + touched * 3.5e-12 : touched * (8.0 * D + 64.0) / 2.0e13;

@@ -38,3 +38,5 @@ def test_complex128_matrices_that_stay_on_the_fp64_pipe():
     on_pipe = N17 * 4 * 9 / 0.5e12
     assert cost([first, shift, last], prec=L.QD_C128) >= on_pipe
     assert cost([shift, last], prec=L.QD_C128) < 0.3 * on_pipe
+    # on a small register a thread's chain of 4 D^2 multiply-adds is what such a launch takes: 25 us
+    assert cost([first, shift, last], dims=(3,) * 8, prec=L.QD_C128) >= 25e-6
