@@ -935,7 +935,9 @@ CostFn cost_for(const qd_reg *r, int plan_kind) {
 
 int segments_for(const qd_reg *r, const std::vector<FuseGate> &fg, int plan_kind,
                  std::vector<std::pair<int, int>> &segs, std::vector<int> &kinds, double *model_cost) {
-    const RegisterShape sh = shape_of(r);
+    RegisterShape sh = shape_of(r);
+    std::map<std::pair<int, int>, bool> fp64_known;
+    sh.fp64_known = &fp64_known;
     const int kmax = r->fuse_kmax;
     const int dmax = r->fuse_dmax > 0 ? r->fuse_dmax : (r->prec == QD_C64 ? kTcMaxD : QD_MAX_D);
     CostFn cost = cost_for(r, plan_kind);

@@ -205,6 +205,76 @@ DenseTableSplit dense_table_split(const std::vector<FuseGate> &gates, int first,
     return d;
 }
 
+namespace {
+// Whether the complex128 tensor cores do not take the product of gates
+// first..last: the same sums as build_block's, gate by gate on the rows that
+// it changes (a planner asks for every candidate segment, 3 us each; 60 gates
+// on 3^12 2^6, exhaustive: 0.25 ms without, 0.90 with build_block, 0.6 so).
+bool product_on_fp64(const std::vector<FuseGate> &gates, int first, int last, const int32_t *dims) {
+    const std::vector<int> qs = union_qudits(gates, first, last);
+    const int64_t Dl = dim_of(qs, dims);
+    if (Dl > kMaxD) return true;
+    const int D = (int)Dl;
+    double re[kMaxD][kMaxD] = {}, im[kMaxD][kMaxD] = {}, nre[kMaxD][kMaxD], nim[kMaxD][kMaxD];
+    for (int i = 0; i < D; ++i) re[i][i] = 1.0;
+    int stride[kMaxD];  // of each block qudit in the local index
+    for (int m = (int)qs.size() - 1, s = 1; m >= 0; s *= dims[qs[m]], --m) stride[m] = s;
+    for (int gi = first; gi <= last; ++gi) {
+        const FuseGate &g = gates[gi];
+        const int n = g.Dact;
+        int off[kMaxD], by_off[kMaxD], moved[kMaxD], nm = 0;  // row of each local index of the gate; rows that change
+        bool of_gate[kMaxD] = {};
+        for (int c = 0; c < n; ++c) {
+            off[c] = 0;
+            int rem = c;
+            for (int a = (int)g.acting.size() - 1; a >= 0; --a) {
+                const int m = (int)(std::find(qs.begin(), qs.end(), g.acting[a]) - qs.begin());
+                off[c] += rem % dims[g.acting[a]] * stride[m];
+                of_gate[m] = true;
+                rem /= dims[g.acting[a]];
+            }
+            by_off[c] = c;
+            bool same = true;
+            for (int k = 0; k < n && same; ++k)
+                same = g.M[2 * (c * n + k)] == (k == c ? 1.0 : 0.0) && g.M[2 * (c * n + k) + 1] == 0.0;
+            if (!same) moved[nm++] = c;
+        }
+        std::sort(by_off, by_off + n, [&](int x, int y) { return off[x] < off[y]; });
+        for (int r = 0; r < D; ++r) {  // the groups: the gate's qudits at level 0
+            bool base = true;
+            for (size_t m = 0; m < qs.size() && base; ++m) base = !of_gate[m] || r / stride[m] % dims[qs[m]] == 0;
+            if (!base) continue;
+            for (int w = 0; w < nm; ++w) {
+                const int i = moved[w];
+                double *__restrict__ xr = nre[w], *__restrict__ xi = nim[w];
+                std::fill(xr, xr + D, 0.0);
+                std::fill(xi, xi + D, 0.0);
+                for (int k = 0; k < n; ++k) {
+                    const double ar = g.M[2 * (i * n + by_off[k])], ai = g.M[2 * (i * n + by_off[k]) + 1];
+                    if (ar == 0.0 && ai == 0.0) continue;
+                    const double *__restrict__ yr = re[r + off[by_off[k]]], *__restrict__ yi = im[r + off[by_off[k]]];
+                    for (int j = 0; j < D; ++j) {
+                        xr[j] += ar * yr[j] - ai * yi[j];
+                        xi[j] += ar * yi[j] + ai * yr[j];
+                    }
+                }
+            }
+            for (int w = 0; w < nm; ++w) {
+                std::copy(nre[w], nre[w] + D, re[r + off[moved[w]]]);
+                std::copy(nim[w], nim[w] + D, im[r + off[moved[w]]]);
+            }
+        }
+    }
+    double M[2 * kMaxD * kMaxD];
+    for (int i = 0; i < D; ++i)
+        for (int j = 0; j < D; ++j) {
+            M[2 * (i * D + j)] = re[i][j];
+            M[2 * (i * D + j) + 1] = im[i][j];
+        }
+    return !tc64_matrix(M, D);
+}
+}  // namespace
+
 double analytic_cost(const RegisterShape &reg, const LaunchFeatures &lf) {
     const double D = std::exp2((double)lf.f[0]);
     const bool c128 = lf.f[9] > 0.5f;
@@ -269,11 +339,12 @@ double segment_cost(const std::vector<FuseGate> &gates, int first, int last, con
         lf.fp64 = g.fp64;
         return cost(lf);
     }
-    // which complex128 kernel takes the product of gates a..b (10 us of host time per gate)
     auto on_fp64 = [&](int a, int b) {
         if (reg.precision == 1) return false;
-        const FuseBlock blk = build_block(gates, a, b, reg.dims);
-        return blk.D > kMaxD || !tc64_matrix(blk.M.data(), blk.D);
+        if (!reg.fp64_known) return product_on_fp64(gates, a, b, reg.dims);
+        const auto known = reg.fp64_known->find({a, b});
+        if (known != reg.fp64_known->end()) return known->second;
+        return reg.fp64_known->emplace(std::make_pair(a, b), product_on_fp64(gates, a, b, reg.dims)).first->second;
     };
     const std::vector<int> s = union_qudits(gates, first, last);
     const int64_t D = dim_of(s, reg.dims);

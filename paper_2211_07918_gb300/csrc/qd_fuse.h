@@ -11,6 +11,8 @@
 #pragma once
 #include <cstdint>
 #include <functional>
+#include <map>
+#include <utility>
 #include <vector>
 
 namespace qd {
@@ -50,6 +52,8 @@ struct RegisterShape {
     int tc_min_d;   // complex64 fused blocks with D >= tc_min_d (or D > 32) run on the tensor cores;
                     // 0: the cost model chooses per block between the CUDA cores and the tensor cores
     int fuse_dmax;  // largest dimension of a fused block
+    // complex128: of the products already formed for this gate list, whether the FP64 pipe keeps them (null: not kept)
+    std::map<std::pair<int, int>, bool> *fp64_known = nullptr;
 };
 
 // Kernel kind of a launch (feature 10).
